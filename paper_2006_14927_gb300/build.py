@@ -24,7 +24,7 @@ BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 
 def debug_requested() -> bool:
     return os.environ.get("CHER_DEBUG", "") == "1"
-SOURCES = ["cher_kernels.cu", "cher_adjoint.cu", "cher_api.cu", "cher_generator.cu", "cher_pack.cu",
+SOURCES = ["cher_hits.cu", "cher_kernels.cu", "cher_adjoint.cu", "cher_api.cu", "cher_generator.cu", "cher_pack.cu",
            "cher_tables.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -44,7 +44,7 @@ def _flags(src: str, debug: bool = False):
         return f + ["-x", "c++"]
     if os.environ.get("CHER_PTXAS_VERBOSE"):
         f += ["-Xptxas", "-v"]
-    if src == "cher_kernels.cu":
+    if src in ("cher_hits.cu", "cher_kernels.cu"):
         # single-precision division and square root by the hardware
         # approximations (<= 2 ulp); double precision is unaffected and the
         # FP64 yield uses explicitly rounded intrinsics

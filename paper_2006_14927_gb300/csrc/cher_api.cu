@@ -39,8 +39,13 @@ struct cher_ctx {
     int32_t *d_cell_start[2] = {nullptr, nullptr}, *d_cell_tel[2] = {nullptr, nullptr};
     float *d_cand32[2] = {nullptr, nullptr};
     double *d_cand64[2] = {nullptr, nullptr};
+    // the hits kernel's bins of telescope centres and table slopes
+    cher::HostBins CB;
+    uint32_t *d_cull_bins = nullptr;
+    float *d_cull_tel = nullptr;
+    double cull_rmax = 0, cull_zmax = 0, ax_sq = 0, ax_sh = 0;
     // scratch: the persistent kernel's tile counter
-    unsigned long long *d_scratch = nullptr;
+    unsigned *d_scratch = nullptr;
     // launch shape
     int block = 128;                      // the autotuner's choice on GB300 for the
     int ctas_per_sm = 8;                  // FP32 path (32 resident warps per SM)
@@ -110,6 +115,10 @@ void free_tables(cher_ctx *c) {
         c->d_cand32[g] = nullptr;
         c->d_cand64[g] = nullptr;
     }
+    cudaFree(c->d_cull_bins);
+    cudaFree(c->d_cull_tel);
+    c->d_cull_bins = nullptr;
+    c->d_cull_tel = nullptr;
     c->d_eta64 = nullptr;
     c->d_eta32 = nullptr;
     c->d_tab64 = c->d_tab32 = nullptr;
@@ -317,6 +326,18 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
         p.grid[g].cand64 = c->d_cand64[g];
     }
     p.q_band = c->q_band;
+    p.cull.tab32 = static_cast<const float2 *>(c->d_tab32);
+    p.cull.ax_sq = static_cast<float>(1.01 * c->ax_sq);
+    p.cull.ax_sh = static_cast<float>(1.01 * c->ax_sh);
+    p.cull.words = c->CB.words;
+    p.cull.x0 = static_cast<float>(c->CB.x0);
+    p.cull.y0 = static_cast<float>(c->CB.y0);
+    p.cull.inv_bx = static_cast<float>(c->CB.inv_bx);
+    p.cull.inv_by = static_cast<float>(c->CB.inv_by);
+    p.cull.r_max = static_cast<float>(c->cull_rmax);
+    p.cull.z_max = static_cast<float>(c->cull_zmax);
+    p.cull.bins = c->d_cull_bins;
+    p.cull.tel = reinterpret_cast<const float4 *>(c->d_cull_tel);
     // the layered thickness, for the production profile
     for (int l = 0; l < 6; ++l) p.atm.hb[l] = c->atm.h_bound[l];
     for (int l = 0; l < 5; ++l) {
@@ -372,33 +393,67 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
     return p;
 }
 
-cher_status launch(cher_ctx *c, cher::KParams &p, bool fp32, int mode, bool persistent,
-                   void *stream) {
-    const int block = (p.disp_k > 0 || p.earth_radius > 0.0) ? cher::kDispBlock : c->block;
-    p.n_tiles = (p.n + block - 1) / block;
-    if (p.n_tiles == 0) return CHER_OK;
-    const size_t smem = cher::kernel_smem_bytes(fp32, block, p);
-    const int kmode = cher::kernel_mode(mode, p) |
-                      (persistent ? cher::occupancy_bits(fp32, block, c->ctas_per_sm) : 0);
-    if (cher::kernel_prepare(fp32, block, kmode, smem) != cudaSuccess) {
+// The launch of a mode: kernel, CTAs, shared memory and, for the hits kernel,
+// the split of the steps over its warps.  `counter` is the word that
+// persistent CTAs (or warps) take work from; NULL: one CTA per tile.  Returns
+// with p.tile_counter = NULL when the launch needs no counter.
+struct Shape {
+    int block = 0, kmode = 0, grid = 0;
+    size_t smem = 0;
+};
+
+cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int ctas_per_sm,
+                 unsigned *counter, Shape &s) {
+    s.block = (p.disp_k > 0 || p.earth_radius > 0.0) ? cher::kDispBlock : c->block;
+    s.kmode = cher::kernel_mode(mode, p);
+    s.smem = cher::kernel_smem_bytes(fp32, s.block, s.kmode, p);
+    p.n_tiles = (p.n + s.block - 1) / s.block;
+    p.tile_counter = nullptr;
+    if (cher::kernel_prepare(fp32, s.block, s.kmode, s.smem) != cudaSuccess) {
         cudaGetLastError();
         return CHER_ERANGE;
     }
-    int grid;
-    if (persistent && c->ctas_per_sm > 0) {
-        const int fit = cher::kernel_max_ctas_per_sm(fp32, block, kmode, smem);
-        const int per_sm = std::max(1, std::min(c->ctas_per_sm, fit));
-        grid = static_cast<int>(std::min<int64_t>(p.n_tiles, int64_t(per_sm) * c->num_sms));
-        p.tile_counter = c->d_scratch;
-        if (cudaMemsetAsync(c->d_scratch, 0, sizeof(unsigned long long),
-                            static_cast<cudaStream_t>(stream)) != cudaSuccess)
-            return CHER_ECUDA;
-    } else {
-        if (p.n_tiles > 0x7fffffff) return CHER_ERANGE;
-        grid = static_cast<int>(p.n_tiles);
-        p.tile_counter = nullptr;
+    const int fit = cher::kernel_max_ctas_per_sm(fp32, s.block, s.kmode, s.smem);
+    const int64_t ctas = int64_t(std::max(1, std::min(ctas_per_sm > 0 ? ctas_per_sm : fit, fit))) *
+                         c->num_sms;
+    int64_t grid = p.n_tiles;
+    if (cher::hits_kernel_serves(s.kmode)) {
+        // groups of 32 steps, fewer where that would leave warps without
+        // work; several groups per claim where there are many
+        const int64_t wpc = s.block / 32, warps = ctas * wpc;
+        p.group = static_cast<int32_t>(std::min<int64_t>(32, std::max<int64_t>(1, (p.n + warps - 1) / warps)));
+        const int64_t groups = (p.n + p.group - 1) / p.group;
+        if (groups > (int64_t(1) << 31)) return CHER_ERANGE;
+        p.n_groups = static_cast<uint32_t>(groups);
+        p.per_claim = counter ? static_cast<int32_t>(std::min<int64_t>(
+                                    8, std::max<int64_t>(1, groups / (warps * 8))))
+                              : 1;
+        const int64_t claims = (groups + p.per_claim - 1) / p.per_claim;
+        grid = (claims + wpc - 1) / wpc;
     }
-    if (cher::kernel_launch(fp32, block, kmode, grid, smem, p, stream) != cudaSuccess) {
+    if (counter && grid > ctas) {
+        grid = ctas;
+        p.tile_counter = counter;
+    } else if (counter && !cher::hits_kernel_serves(s.kmode)) {
+        p.tile_counter = counter;
+    }
+    if (grid > 0x7fffffff || (p.tile_counter && p.n_tiles > 0xf0000000ll)) return CHER_ERANGE;
+    s.grid = static_cast<int>(grid);
+    return CHER_OK;
+}
+
+cher_status launch(cher_ctx *c, cher::KParams &p, bool fp32, int mode, bool persistent,
+                   void *stream) {
+    if (p.n == 0) return CHER_OK;
+    Shape s;
+    const bool counted = persistent && c->ctas_per_sm > 0;
+    const cher_status r = plan(c, p, fp32, mode, counted ? c->ctas_per_sm : 0,
+                               counted ? c->d_scratch : nullptr, s);
+    if (r != CHER_OK) return r;
+    if (p.tile_counter && cudaMemsetAsync(p.tile_counter, 0, sizeof(unsigned),
+                                          static_cast<cudaStream_t>(stream)) != cudaSuccess)
+        return CHER_ECUDA;
+    if (cher::kernel_launch(fp32, s.block, s.kmode, s.grid, s.smem, p, stream) != cudaSuccess) {
         cudaGetLastError();
         return CHER_ECUDA;
     }
@@ -580,6 +635,20 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
             tel32[4 * k + m] = static_cast<float>(v[m]);
         }
     }
+    // the telescopes for the hits kernel's bound (radii rounded up)
+    cher::build_center_bins(c->tel.data(), static_cast<int32_t>(nt), c->CB);
+    std::vector<float> ctel(nt * 4);
+    c->cull_rmax = c->cull_zmax = 0.0;
+    for (size_t m = 0; m < nt; ++m) {
+        const cher_telescope &q = c->tel[m];
+        ctel[4 * m] = static_cast<float>(q.x);
+        ctel[4 * m + 1] = static_cast<float>(q.y);
+        ctel[4 * m + 2] = static_cast<float>(q.z);
+        ctel[4 * m + 3] = static_cast<float>(q.r * (1.0 + 1e-6));
+        c->cull_rmax = std::max(c->cull_rmax, q.r * (1.0 + 1e-6));
+        c->cull_zmax = std::max(c->cull_zmax, std::fabs(q.z) * (1.0 + 1e-6));
+    }
+    cher::table_slopes(c->T, c->ax_sq, c->ax_sh);
     cher_status r;
     double *d_tab64 = nullptr;
     float *d_tab32 = nullptr, *d_tel32 = nullptr;
@@ -590,6 +659,8 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
         (r = upload(&d_tab32, t32.data(), t32.size())) != CHER_OK ||
         (r = upload(&d_tel64, tel64.data(), tel64.size())) != CHER_OK ||
         (r = upload(&d_tel32, tel32.data(), tel32.size())) != CHER_OK ||
+        (r = upload(&c->d_cull_bins, c->CB.masks.data(), c->CB.masks.size())) != CHER_OK ||
+        (r = upload(&c->d_cull_tel, ctel.data(), ctel.size())) != CHER_OK ||
         (r = upload_grid(c, 0)) != CHER_OK || (r = upload_grid(c, 1)) != CHER_OK) {
         c->d_tab64 = d_tab64;
         c->d_tab32 = d_tab32;
@@ -1451,7 +1522,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 void *g_static_addr[kMaxDevices] = {};
 
-cher_status static_scratch(int device, unsigned long long **out) {
+cher_status static_scratch(int device, unsigned **out) {
     if (device < 0 || device >= kMaxDevices) return CHER_ERANGE;
     std::lock_guard<std::mutex> lock(g_static_mutex);
     if (!g_static_addr[device]) {
@@ -1462,7 +1533,7 @@ cher_status static_scratch(int device, unsigned long long **out) {
         }
         g_static_addr[device] = ptr;
     }
-    *out = static_cast<unsigned long long *>(g_static_addr[device]);
+    *out = static_cast<unsigned *>(g_static_addr[device]);
     return CHER_OK;
 }
 
@@ -1490,7 +1561,7 @@ extern "C" cher_status cher_generate_propagate_noalloc(cher_ctx *c, const cher_t
     // allocates: with it active this call would drop them where the regular
     // entry point propagates them, so it refuses instead
     if (c->fb_deg > c->tab_zen && c->earth_radius == 0.0) return CHER_EINVAL;
-    unsigned long long *scratch = nullptr;
+    unsigned *scratch = nullptr;
     cher_status s = static_scratch(c->device, &scratch);
     if (s != CHER_OK) return s;
 
@@ -1508,25 +1579,16 @@ extern "C" cher_status cher_generate_propagate_noalloc(cher_ctx *c, const cher_t
     p.cap = out->cap_per_tel;
     p.count = out->count;
     p.stats = out->stats;
-    const int block = (p.disp_k > 0 || p.earth_radius > 0.0) ? cher::kDispBlock : c->block;
-    p.n_tiles = (p.n + block - 1) / block;
-    if (p.n_tiles == 0) return CHER_OK;
-    const size_t smem = cher::kernel_smem_bytes(fp32, block, p);
-    const int kmode = cher::kernel_mode(cher::MODE_HITS, p) |
-                      cher::occupancy_bits(fp32, block, c->ctas_per_sm);
-    if (cher::kernel_prepare(fp32, block, kmode, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return CHER_ERANGE;
-    }
-    const int fit = cher::kernel_max_ctas_per_sm(fp32, block, kmode, smem);
-    const int per_sm = std::max(1, std::min(c->ctas_per_sm > 0 ? c->ctas_per_sm : 1, fit));
-    const int grid =
-        static_cast<int>(std::min<int64_t>(p.n_tiles, int64_t(per_sm) * c->num_sms));
+    if (p.n == 0) return CHER_OK;
+    Shape sh;
+    s = plan(c, p, fp32, cher::MODE_HITS, std::max(1, c->ctas_per_sm), scratch, sh);
+    if (s != CHER_OK) return s;
     // the array keeps the previous call's contents: clear the counter first
-    k_clear_static_scratch<<<1, 32, 0, st>>>(static_cast<int>(need / sizeof(unsigned long long)));
-    if (cudaGetLastError() != cudaSuccess) return CHER_ECUDA;
-    p.tile_counter = scratch;
-    if (cher::kernel_launch(fp32, block, kmode, grid, smem, p, stream) != cudaSuccess) {
+    if (p.tile_counter) {
+        k_clear_static_scratch<<<1, 32, 0, st>>>(static_cast<int>(need / sizeof(unsigned long long)));
+        if (cudaGetLastError() != cudaSuccess) return CHER_ECUDA;
+    }
+    if (cher::kernel_launch(fp32, sh.block, sh.kmode, sh.grid, sh.smem, p, stream) != cudaSuccess) {
         cudaGetLastError();
         return CHER_ECUDA;
     }

@@ -151,8 +151,9 @@ __device__ __forceinline__ bool finite_r(R v) {
 
 template <class R>
 __device__ __forceinline__ bool step_valid(const KParams &p, int64_t i) {
-    return finite_d(__ldg(p.x0 + i)) && finite_d(__ldg(p.y0 + i)) && finite_d(__ldg(p.t0 + i)) &&
-           finite_r<R>(__ldg(static_cast<const R *>(p.ux) + i)) &&
+    // (no short circuit: the loads go out together)
+    return finite_d(__ldg(p.x0 + i)) & finite_d(__ldg(p.y0 + i)) & finite_d(__ldg(p.t0 + i)) &
+           finite_r<R>(__ldg(static_cast<const R *>(p.ux) + i)) &
            finite_r<R>(__ldg(static_cast<const R *>(p.uy) + i));
 }
 

@@ -26,6 +26,7 @@ enum : int32_t {
 };
 
 constexpr int kMaxCandPerCell = 32;   // telescope candidates in one grid cell
+constexpr int kCullBins = 128;        // bins of the telescopes' centres per axis
 constexpr int kDispMax = 9;           // nodes of a wavelength-dependent index
 
 // Host-side tables, all FP64 (step a0).
@@ -61,6 +62,15 @@ cher_status build_tables(const cher_atmosphere &atm, double h_obs, int32_t n_fin
 double eta_lookup(const HostTables &t, double h);
 cher_status build_grid(const cher_telescope *tel, int32_t n_tel, double theta_max,
                        HostGrid &g);
+// Prefix masks of the telescopes' centres over kCullBins bins per axis
+// (KParams::cull), and the largest slopes of ax over the table's cells.
+struct HostBins {
+    int32_t words = 0;
+    double x0 = 0, y0 = 0, inv_bx = 0, inv_by = 0;
+    std::vector<uint32_t> masks;          // [2][kCullBins + 1][words]
+};
+void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b);
+void table_slopes(const HostTables &T, double &per_q, double &per_h);
 // Adjoint support: d eta(h) / d p and the refraction-table sensitivities
 // [H][Z][20] = {d ax / d p (10), d al / d p (10)}, p = b_0..b_4, c_0..c_4.
 void eta_sensitivity(const cher_atmosphere &atm, double h, double *d);
@@ -117,6 +127,20 @@ struct KParams {
         const void *cand64;               // double4 per entry
     } grid[2];
     double q_band;
+    // the hits kernel's bound of the azimuths that reach a sphere: the FP32
+    // node table (flat layers), the largest slopes of its horizontal
+    // correction (per sin^2 of the zenith, per metre of height), the
+    // telescopes (float4 x, y, z, r) with the largest radius and height, and
+    // for boxes of their centres the prefix masks of kCullBins bins per axis:
+    // word w of entry b holds the telescopes 32 w .. 32 w + 31 in bins < b
+    struct Cull {
+        const float2 *tab32;
+        float ax_sq, ax_sh;
+        int words;
+        float x0, y0, inv_bx, inv_by, r_max, z_max, r_cut;
+        const uint32_t *bins;             // [2][kCullBins + 1][words], x then y
+        const float4 *tel;                // [n_tel]
+    } cull;
     // outputs
     void *pos, *tim;
     uint64_t *key;
@@ -130,8 +154,11 @@ struct KParams {
     int32_t *y_nb;
     double *y_w;
     // scheduling
-    unsigned long long *tile_counter;     // NULL: one CTA per tile
+    unsigned *tile_counter;               // NULL: one CTA per tile
     int64_t n_tiles;
+    // the hits kernel's warps take `per_claim` groups of `group` steps at once
+    int32_t group, per_claim;
+    uint32_t n_groups;
     // adjoint screening: frozen bunch counts, list of (step, bunch) pairs
     // that land within the read-out radius of a telescope centre
     const int32_t *nb_frozen;
@@ -236,15 +263,6 @@ constexpr int kFbBit = 8;
 // only; the curved atmosphere without the beyond-table fallback)
 constexpr int kDispBit = 16;
 constexpr int kCurvBit = 32;
-// The plain FP32 hits kernel also comes in builds for more resident CTAs per
-// SM (128 threads each, fewer registers per thread): 9 or 10; the launch
-// shape's CTAs per SM picks one (kOccShift: 2 bits of the mode word).
-constexpr int kOccShift = 6;
-constexpr int kOccMask = 3 << kOccShift;
-inline int occupancy_bits(bool fp32, int block, int ctas_per_sm) {
-    if (!fp32 || block != 128 || ctas_per_sm <= 8) return 0;
-    return (ctas_per_sm <= 9 ? 1 : 2) << kOccShift;
-}
 constexpr int kDispBlock = 128;
 inline int kernel_mode(int mode, const KParams &p) {
     int m = mode;
@@ -263,8 +281,14 @@ size_t fallback_record_bytes(bool fp32);
 // The 12-point Gauss-Legendre rule on [-1, 1] (host).
 void gauss_legendre12(double *x, double *w);
 
+// The hits kernel of flat layers and the screening pass (cher_hits.cu): the
+// modes it serves, its instantiation and its shared memory per CTA.
+bool hits_kernel_serves(int mode);
+const void *hits_kernel(bool fp32, int mode);
+size_t hits_smem_bytes(bool fp32, int mode, int block);
+
 // Launchers (cher_kernels.cu).  fp32 selects CHER_FP32_BULK.
-size_t kernel_smem_bytes(bool fp32, int block, const KParams &p);
+size_t kernel_smem_bytes(bool fp32, int block, int mode, const KParams &p);
 // Device step generator (cher_generator.cu): per-shower constants in float.
 struct GenShower {
     float ax, ay, az;            // axis (downward)

@@ -571,6 +571,44 @@ cher_status build_grid(const cher_telescope *tel, int32_t n_tel, double theta_ma
     return CHER_ERANGE;
 }
 
+void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
+    b.words = (n_tel + 31) / 32;
+    b.masks.assign(2 * size_t(kCullBins + 1) * b.words, 0u);
+    for (int axis = 0; axis < 2; ++axis) {
+        double lo = 1e300, hi = -1e300;
+        for (int k = 0; k < n_tel; ++k) {
+            const double v = axis ? tel[k].y : tel[k].x;
+            lo = std::min(lo, v);
+            hi = std::max(hi, v);
+        }
+        // room on both sides for single-precision bin indices
+        const double mag = 1.0 + 1e-5 * std::max(std::fabs(lo), std::fabs(hi));
+        lo -= mag;
+        const double inv = kCullBins / (hi + mag - lo);
+        (axis ? b.y0 : b.x0) = lo;
+        (axis ? b.inv_by : b.inv_bx) = inv;
+        uint32_t *m = b.masks.data() + axis * size_t(kCullBins + 1) * b.words;
+        for (int k = 0; k < n_tel; ++k) {
+            const int bin = std::min(kCullBins - 1,
+                                     static_cast<int>(((axis ? tel[k].y : tel[k].x) - lo) * inv));
+            for (int e = bin + 1; e <= kCullBins; ++e)
+                m[size_t(e) * b.words + k / 32] |= 1u << (k % 32);
+        }
+    }
+}
+
+void table_slopes(const HostTables &T, double &per_q, double &per_h) {
+    per_q = per_h = 0.0;
+    for (int j = 0; j < T.H; ++j)
+        for (int k = 0; k < T.Z; ++k) {
+            const size_t a = static_cast<size_t>(j) * T.Z + k;
+            if (k + 1 < T.Z)
+                per_q = std::max(per_q, std::fabs(T.ax[a + 1] - T.ax[a]) * T.inv_dq);
+            if (j + 1 < T.H)
+                per_h = std::max(per_h, std::fabs(T.ax[a + T.Z] - T.ax[a]) * T.inv_dht);
+        }
+}
+
 // Greisen profile of a shower of y = ln(E0 / E_c), up to a constant factor,
 // and its CDF on n_cdf uniform nodes of [0, t_g], normalised to 1 (the
 // device step generator inverts it); Gauss-Legendre on each node interval.
