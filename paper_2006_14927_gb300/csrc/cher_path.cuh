@@ -113,7 +113,9 @@ __device__ __forceinline__ bool screen_yield(const KParams &p, bool others_valid
     const float np1 = 1.0f + eta, np1sq = np1 * np1;
     const float a = eta * (2.0f + eta);
     const float A = a * gam2;
-    const float num = A - np1sq;
+    // (one rounding, written out: left to the compiler, the instantiations of
+    // the kernels would not all fuse it)
+    const float num = __fmaf_rn(a, gam2, -np1sq);
     const float bg2 = g * (2.0f + g);
     const float den = bg2 * np1sq;
     const float s2 = num / den;
@@ -314,7 +316,7 @@ __device__ __forceinline__ bool screen_yield_disp(const KParams &p, bool others_
                 const float ea = eta * ka, eb = eta * kb;
                 const float ee = (ea + eb) + ea * eb;
                 const float B = 1.0f + ee, A = ee * gam2;
-                const float num = A - B, den = bg2 * B;
+                const float num = __fmaf_rn(ee, gam2, -B), den = bg2 * B;
                 const float S = num / den;
                 const float d_e = (ka + kb) * (1.0f + ee) * d_eta + 4.0f * u * ee;
                 const float d_A = gam2 * (d_e + 10.0f * u * ee);
