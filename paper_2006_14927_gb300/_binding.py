@@ -575,8 +575,8 @@ class Context:
         """Smoothed photon density D_k and mean arrival time Tbar_k (device f64)."""
         torch = _torch()
         dev = dev_tracks["x0"].device
-        D = torch.zeros(self.n_tel, dtype=torch.float64, device=dev)
-        T = torch.zeros(self.n_tel, dtype=torch.float64, device=dev)
+        D = torch.empty(self.n_tel, dtype=torch.float64, device=dev)     # (all written)
+        T = torch.empty(self.n_tel, dtype=torch.float64, device=dev)
         t = self.tracks_struct(dev_tracks, track_base)
         _check(lib().cher_density(self._h, ctypes.byref(t), ctypes.c_uint64(seed), int(precision),
                                   float(sigma),
@@ -591,8 +591,8 @@ class Context:
         torch = _torch()
         dev = dev_tracks["x0"].device
         n = int(dev_tracks["x0"].numel())
-        ga = torch.zeros(15, dtype=torch.float64, device=dev)
-        gt = torch.zeros((6, n), dtype=torch.float64, device=dev)
+        ga = torch.empty(15, dtype=torch.float64, device=dev)            # (zeroed by the call)
+        gt = torch.empty((6, n), dtype=torch.float64, device=dev)
         gD = torch.as_tensor(dL_dD, dtype=torch.float64, device=dev).contiguous()
         gT = torch.as_tensor(dL_dT, dtype=torch.float64, device=dev).contiguous()
         t = self.tracks_struct(dev_tracks, track_base)

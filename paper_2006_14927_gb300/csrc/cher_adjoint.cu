@@ -24,6 +24,7 @@
 // depend on a_i, whose gradient is exactly zero.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -170,10 +171,10 @@ __device__ __forceinline__ void eta_sens(const AdjParams &a, int k, double f, do
         int i = 0;
         while (i < 4 && h >= a.hb[i + 1]) ++i;
         const double e = __ldg(a.k.eta64 + kk) * wgt;
-        d[i] += e / a.b[i];
-        d[a.layer0] -= e / a.b[a.layer0];
-        d[5 + i] += e * (h - a.c[i]) / (a.c[i] * a.c[i]);
-        d[5 + a.layer0] += e / a.c[a.layer0];
+        d[i] += e * a.inv_b[i];
+        d[a.layer0] -= e * a.inv_b[a.layer0];
+        d[5 + i] += e * ((h - a.c[i]) * a.inv_c[i] * a.inv_c[i]);
+        d[5 + a.layer0] += e * a.inv_c[a.layer0];
     }
 }
 
@@ -337,8 +338,15 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
 // shower crowd around a handful of telescopes.
 constexpr int kSmemTel = 512;     // telescopes whose S, U are combined in smem
 
+// One warp per CTA: a list of some thousand bunches is a long chain of FP64
+// work per thread (GB300: 2 FP64 lanes per SM and clock), so it is spread over
+// as many SMs as it has warps.  On the 300 GeV read-out (5e3 bunches listed):
+// FP32 recomputation, value pass 37.5 -> PAIRS0 us and gradient pass 120 ->
+// PAIRS1 us against CTAs of 128.
+constexpr int kPairBlock = 32;
+
 template <class T, int MODE>
-__global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
+__global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
     __shared__ double s_sum[MODE == 0 ? 2 * kSmemTel : 10];
     const int n_tel = A.k.n_tel;
     const bool smem_su = MODE == 0 && n_tel <= kSmemTel;
@@ -346,7 +354,10 @@ __global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
     for (int q = threadIdx.x; q < n_red; q += blockDim.x) s_sum[q] = 0.0;
     __syncthreads();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < A.n_list;
+    const unsigned long long listed = *A.count;
+    const int64_t n_list = static_cast<int64_t>(
+        listed < static_cast<unsigned long long>(A.list_cap) ? listed : A.list_cap);
+    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n_list;
          e += stride) {
         const uint64_t ent = A.list[e];
         const int64_t i = static_cast<int64_t>(ent >> 32);
@@ -356,12 +367,16 @@ __global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
         const double X = o.X.v, Y = o.Y.v, t = o.t.v, w = o.w.v;
         double gX = 0, gY = 0, gt = 0, gw = 0;
         bool any = false;
+        const float Xf = static_cast<float>(o.X.v), Yf = static_cast<float>(o.Y.v);
         for (int k = 0; k < A.k.n_tel; ++k) {
+            // most telescopes are out of reach: seen in FP32, with room for
+            // its rounding
+            const float4 C = __ldg(A.k.cull.tel + k);
+            if (!(fabsf(Xf - C.x) < A.reach && fabsf(Yf - C.y) < A.reach)) continue;
             double tx, ty;
             if constexpr (std::is_same<T, float>::value) {
-                const float4 Tt = __ldg(static_cast<const float4 *>(A.k.tel) + k);
-                tx = Tt.x;
-                ty = Tt.y;
+                tx = C.x;
+                ty = C.y;
             } else {
                 const double2 Tt = __ldg(static_cast<const double2 *>(A.k.tel) + 2 * k);
                 tx = Tt.x;
@@ -405,10 +420,9 @@ __global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
                         gt * static_cast<double>(o.t.d[c]) + gw * static_cast<double>(o.w.d[c]);
             for (int m = 0; m < 6; ++m) atomicAdd(A.grad_tracks + m * A.k.n + i, gl[m]);
             // atmosphere: the five channels through their sensitivities
-            double dm[10], de[10], dob[10];
+            double dm[10], de[10];
             eta_sens(A, o.km, static_cast<double>(o.fm), dm);
             eta_sens(A, o.ke, static_cast<double>(o.fe), de);
-            eta_sens(A, A.ko, A.fo, dob);
             const double *s00 = A.sens + (static_cast<size_t>(o.jj) * A.k.Z + o.kk) * 20;
             const double *s01 = s00 + 20;
             const double *s10 = s00 + static_cast<size_t>(A.k.Z) * 20;
@@ -423,7 +437,7 @@ __global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
                     tab[m] = v0 + bb * (v1 - v0);
                 }
                 const double gp = gl[C_ETA_M] * dm[q] + gl[C_ETA_E] * de[q] +
-                                  gl[C_ETA_O] * dob[q] + gl[C_AX] * tab[0] + gl[C_AL] * tab[1];
+                                  gl[C_ETA_O] * A.dob[q] + gl[C_AX] * tab[0] + gl[C_AL] * tab[1];
                 atomicAdd(s_sum + q, gp);            // b_i at 5 + i, c_i at 10 + i
             }
         }
@@ -439,21 +453,38 @@ __global__ void __launch_bounds__(128) k_adj_pairs(const AdjParams A) {
     }
 }
 
+// D_k = S_k and Tbar_k = U_k / S_k (0 where no bunch came near).
+__global__ void k_readout(const double *S, const double *U, double *D, double *T, int n_tel) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n_tel) return;
+    const double s = S[k];
+    if (D) D[k] = s;
+    if (T) T[k] = s > 0.0 ? U[k] / s : 0.0;
+}
+
 template <class T, int MODE>
-cudaError_t launch_pairs(const AdjParams &A, void *stream) {
-    if (A.n_list == 0) return cudaSuccess;
-    const int block = 128;
-    const int64_t want = (A.n_list + block - 1) / block;
-    const int grid = static_cast<int>(want < 4096 ? want : 4096);
-    k_adj_pairs<T, MODE><<<grid, block, 0, static_cast<cudaStream_t>(stream)>>>(A);
+cudaError_t launch_pairs(const AdjParams &A, int num_sms, void *stream) {
+    // (the list's length is on the device: warps without an entry just end)
+    const int64_t want = (A.list_cap + kPairBlock - 1) / kPairBlock;
+    const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, num_sms * 16)));
+    k_adj_pairs<T, MODE><<<grid, kPairBlock, 0, static_cast<cudaStream_t>(stream)>>>(A);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t adjoint_pairs(bool fp32, int mode, const AdjParams &A, void *stream) {
-    if (fp32) return mode == 0 ? launch_pairs<float, 0>(A, stream) : launch_pairs<float, 1>(A, stream);
-    return mode == 0 ? launch_pairs<double, 0>(A, stream) : launch_pairs<double, 1>(A, stream);
+cudaError_t adjoint_pairs(bool fp32, int mode, const AdjParams &A, int num_sms, void *stream) {
+    if (fp32)
+        return mode == 0 ? launch_pairs<float, 0>(A, num_sms, stream)
+                         : launch_pairs<float, 1>(A, num_sms, stream);
+    return mode == 0 ? launch_pairs<double, 0>(A, num_sms, stream)
+                     : launch_pairs<double, 1>(A, num_sms, stream);
+}
+
+cudaError_t readout_values(const double *S, const double *U, double *D, double *T, int n_tel,
+                           void *stream) {
+    k_readout<<<(n_tel + 127) / 128, 128, 0, static_cast<cudaStream_t>(stream)>>>(S, U, D, T, n_tel);
+    return cudaGetLastError();
 }
 
 }  // namespace cher

@@ -55,12 +55,11 @@ struct cher_ctx {
     // adjoint: sensitivity tables and scratch, allocated on first use
     double *d_sens = nullptr;
     int32_t *d_nb = nullptr;
-    double *d_w = nullptr;
     int64_t nb_cap = 0;
     uint64_t *d_list = nullptr;
     int64_t list_cap = 0;
-    unsigned long long *d_list_count = nullptr;
-    double *d_SU = nullptr;
+    double *d_SU = nullptr;               // S, U per telescope, then the list's count
+    unsigned long long *h_count = nullptr;   // (pinned) where the host reads it
     // atmospheric transmission table (both precisions), NULL when off
     double *d_trans64 = nullptr;
     float *d_trans32 = nullptr;
@@ -140,15 +139,13 @@ void free_dispersion_tables(cher_ctx *c) {
 
 void free_adjoint_scratch(cher_ctx *c) {
     cudaFree(c->d_nb);
-    cudaFree(c->d_w);
     cudaFree(c->d_list);
-    cudaFree(c->d_list_count);
     cudaFree(c->d_SU);
+    cudaFreeHost(c->h_count);
     c->d_nb = nullptr;
-    c->d_w = nullptr;
     c->d_list = nullptr;
-    c->d_list_count = nullptr;
     c->d_SU = nullptr;
+    c->h_count = nullptr;
     c->nb_cap = c->list_cap = 0;
 }
 
@@ -1279,112 +1276,97 @@ cher_status readout(cher_ctx *c, const cher_tracks *t, uint64_t seed, cher_preci
         if ((r = cher::build_sensitivity(c->atm, c->h_obs, c->T, sv)) != CHER_OK) return r;
         if ((r = upload(&c->d_sens, sv.data(), sv.size())) != CHER_OK) return r;
     }
-    int64_t cap_tmp = c->nb_cap;
-    if ((r = grow(&c->d_nb, cap_tmp, t->n)) != CHER_OK) return r;
-    int64_t cap_w = c->nb_cap;
-    if ((r = grow(&c->d_w, cap_w, t->n)) != CHER_OK) return r;
-    c->nb_cap = std::max(cap_tmp, cap_w);
-    int64_t one = c->d_list_count ? 1 : 0;
-    if ((r = grow(&c->d_list_count, one, 1)) != CHER_OK) return r;
-    int64_t su = c->d_SU ? 2 * n_tel : 0;
-    if ((r = grow(&c->d_SU, su, 2 * n_tel)) != CHER_OK) return r;
+    if ((r = grow(&c->d_nb, c->nb_cap, t->n)) != CHER_OK) return r;
+    int64_t su = c->d_SU ? 2 * n_tel + 1 : 0;
+    if ((r = grow(&c->d_SU, su, 2 * n_tel + 1)) != CHER_OK) return r;
+    if (!c->h_count) {
+        void *h = nullptr;
+        if (cudaHostAlloc(&h, sizeof(unsigned long long), cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            return CHER_ENOMEM;
+        }
+        c->h_count = static_cast<unsigned long long *>(h);
+    }
     if (!c->d_list && (r = grow(&c->d_list, c->list_cap, std::max<int64_t>(1 << 16, t->n / 8))) != CHER_OK)
         return r;
-    // frozen bunch counts: the caller's, or this call's yield
-    const int32_t *nb = nb_frozen;
-    if (!nb) {
-        cher::KParams p = base_params(c, t, seed, fp32);
-        p.y_nb = c->d_nb;
-        p.y_w = c->d_w;
-        if ((r = launch(c, p, fp32, cher::MODE_YIELD, false, stream)) != CHER_OK) return r;
-        nb = c->d_nb;
-    }
-    // screen: list the bunches within 6 sigma (plus a margin) of a centre
+    unsigned long long *count = reinterpret_cast<unsigned long long *>(c->d_SU + 2 * n_tel);
+    // bunches within 6 sigma (plus a margin) of a centre are listed; their
+    // counts are the caller's frozen ones, or this pass's own
     const double rscreen = 6.0 * sigma + 0.05;
-    unsigned long long count = 0;
-    for (int attempt = 0; attempt < 3; ++attempt) {
-        if (cudaMemsetAsync(c->d_list_count, 0, sizeof(unsigned long long), st) != cudaSuccess)
-            return CHER_ECUDA;
-        cher::KParams p = base_params(c, t, seed, fp32);
-        p.nb_frozen = nb;
-        p.list = c->d_list;
-        p.list_count = c->d_list_count;
-        p.list_cap = c->list_cap;
-        p.rcut2 = rscreen * rscreen;
-        cher::fill_float_constants(p);
-        if ((r = launch(c, p, fp32, cher::MODE_SCREEN, false, stream)) != CHER_OK) return r;
-        if (cudaMemcpyAsync(&count, c->d_list_count, sizeof(count), cudaMemcpyDeviceToHost, st) !=
-                cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return CHER_ECUDA;
-        if (static_cast<int64_t>(count) <= c->list_cap) break;
-        if ((r = grow(&c->d_list, c->list_cap, static_cast<int64_t>(count) + count / 4 + 1024)) !=
-            CHER_OK)
-            return r;
-    }
-    if (static_cast<int64_t>(count) > c->list_cap) return CHER_ERANGE;
-    // the pass over the listed bunches: sums, then gradients
+    cher::KParams p = base_params(c, t, seed, fp32);
+    p.nb_frozen = nb_frozen;
+    p.y_nb = c->d_nb;
+    p.list_count = count;
+    p.rcut2 = rscreen * rscreen;
+    cher::fill_float_constants(p);
     cher::AdjParams A;
     std::memset(&A, 0, sizeof(A));
     A.k = base_params(c, t, seed, fp32);
-    A.list = c->d_list;
-    A.n_list = static_cast<int64_t>(count);
-    A.nb = nb;
+    A.count = count;
+    A.nb = nb_frozen ? nb_frozen : c->d_nb;
     A.sigma = sigma;
     A.inv_2s2 = 1.0 / (2.0 * sigma * sigma);
     A.norm = 1.0 / (2.0 * cher::kPi * sigma * sigma);
     A.rcut2 = 36.0 * sigma * sigma;
+    double far = 0.0;
+    for (const cher_telescope &q : c->tel) far = std::max({far, std::fabs(q.x), std::fabs(q.y)});
+    A.reach = static_cast<float>(6.0 * sigma * 1.0001 + 1e-3 + 1e-6 * far);
     A.S = c->d_SU;
     A.U = c->d_SU + n_tel;
     A.sens = c->d_sens;
     for (int i = 0; i < 6; ++i) A.hb[i] = c->atm.h_bound[i];
     for (int i = 0; i < 5; ++i) {
-        A.b[i] = c->atm.b[i];
         A.c[i] = c->atm.c[i];
+        A.inv_b[i] = 1.0 / c->atm.b[i];
+        A.inv_c[i] = 1.0 / c->atm.c[i];
     }
     A.layer0 = 0;
     while (A.layer0 < 4 && 0.0 >= A.hb[A.layer0 + 1]) ++A.layer0;
     A.dh_fine = c->T.dh;
     {
-        double hc = std::min(std::max(c->h_obs, 0.0), c->T.h_max);
+        // d eta(h_obs) / d p at its place in the fine table, like the values
+        const double hc = std::min(std::max(c->h_obs, 0.0), c->T.h_max);
         const double x = hc * c->T.inv_dh;
-        int k = static_cast<int>(x);
-        if (k > c->T.n_fine - 2) k = c->T.n_fine - 2;
-        A.ko = k;
-        A.fo = x - k;
-    }
-    if (cudaMemsetAsync(c->d_SU, 0, 2 * n_tel * sizeof(double), st) != cudaSuccess)
-        return CHER_ECUDA;
-    if (cher::adjoint_pairs(fp32, 0, A, stream) != cudaSuccess) return CHER_ECUDA;
-    if (D || Tbar) {
-        std::vector<double> su(2 * n_tel), d(n_tel), tb(n_tel);
-        if (cudaMemcpyAsync(su.data(), c->d_SU, su.size() * sizeof(double),
-                            cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return CHER_ECUDA;
-        for (int k = 0; k < n_tel; ++k) {
-            d[k] = su[k];
-            tb[k] = su[k] > 0.0 ? su[n_tel + k] / su[k] : 0.0;
+        const int k = std::min(static_cast<int>(x), c->T.n_fine - 2);
+        for (int side = 0; side < 2; ++side) {
+            double d[10];
+            cher::eta_sensitivity(c->atm, static_cast<double>(k + side) * c->T.dh, d);
+            for (int q = 0; q < 10; ++q) A.dob[q] += (side ? x - k : 1.0 - (x - k)) * d[q];
         }
-        if ((D && cudaMemcpyAsync(D, d.data(), n_tel * sizeof(double), cudaMemcpyHostToDevice,
-                                  st) != cudaSuccess) ||
-            (Tbar && cudaMemcpyAsync(Tbar, tb.data(), n_tel * sizeof(double),
-                                     cudaMemcpyHostToDevice, st) != cudaSuccess) ||
+    }
+    A.gD = gD;
+    A.gT = gT;
+    A.grad_atm = grad_atm;
+    A.grad_tracks = grad_tracks;
+    // everything goes out before the host looks at the list's length; where
+    // the list was too short (a first call), it grows and all is done again
+    for (int attempt = 0; attempt < 3; ++attempt) {
+        p.list = c->d_list;
+        p.list_cap = c->list_cap;
+        A.list = c->d_list;
+        A.list_cap = c->list_cap;
+        if (cudaMemsetAsync(c->d_SU, 0, (2 * n_tel + 1) * sizeof(double), st) != cudaSuccess)
+            return CHER_ECUDA;
+        if ((r = launch(c, p, fp32, cher::MODE_SCREEN, false, stream)) != CHER_OK) return r;
+        if (cher::adjoint_pairs(fp32, 0, A, c->num_sms, stream) != cudaSuccess) return CHER_ECUDA;
+        if ((D || Tbar) && cher::readout_values(A.S, A.U, D, Tbar, n_tel, stream) != cudaSuccess)
+            return CHER_ECUDA;
+        if (grad_atm) {
+            if (cudaMemsetAsync(grad_atm, 0, 15 * sizeof(double), st) != cudaSuccess ||
+                (t->n > 0 && cudaMemsetAsync(grad_tracks, 0, 6 * static_cast<size_t>(t->n) * sizeof(double),
+                                             st) != cudaSuccess))
+                return CHER_ECUDA;
+            if (cher::adjoint_pairs(fp32, 1, A, c->num_sms, stream) != cudaSuccess) return CHER_ECUDA;
+        }
+        if (cudaMemcpyAsync(c->h_count, count, sizeof(*count), cudaMemcpyDeviceToHost, st) !=
+                cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return CHER_ECUDA;
+        const int64_t listed = static_cast<int64_t>(*c->h_count);
+        if (listed <= c->list_cap) return CHER_OK;
+        if ((r = grow(&c->d_list, c->list_cap, listed + listed / 4 + 1024)) != CHER_OK) return r;
     }
-    if (grad_atm) {
-        if (cudaMemsetAsync(grad_atm, 0, 15 * sizeof(double), st) != cudaSuccess ||
-            cudaMemsetAsync(grad_tracks, 0, 6 * static_cast<size_t>(t->n) * sizeof(double), st) !=
-                cudaSuccess)
-            return CHER_ECUDA;
-        A.gD = gD;
-        A.gT = gT;
-        A.grad_atm = grad_atm;
-        A.grad_tracks = grad_tracks;
-        if (cher::adjoint_pairs(fp32, 1, A, stream) != cudaSuccess) return CHER_ECUDA;
-    }
-    return CHER_OK;
+    return CHER_ERANGE;
 }
 
 }  // namespace

@@ -409,8 +409,12 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 if (!open) {
                     if constexpr (MODE == MODE_SCREEN) {
                         // the adjoint freezes the sub-step structure
-                        const int nf = __ldg(p.nb_frozen + i);
-                        y.nb = (y.s2 > 0.0 && nf > 0) ? nf : 0;
+                        if (p.nb_frozen) {
+                            const int nf = __ldg(p.nb_frozen + i);
+                            y.nb = (y.s2 > 0.0 && nf > 0) ? nf : 0;
+                        } else {
+                            p.y_nb[i] = y.nb;
+                        }
                     }
                     if constexpr (MODE == MODE_HITS) {
                         if (p.prof && y.nb > 0) profile_call<R>(p, i, static_cast<R>(y.N));

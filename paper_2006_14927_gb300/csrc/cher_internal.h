@@ -159,7 +159,8 @@ struct KParams {
     // the hits kernel's warps take `per_claim` groups of `group` steps at once
     int32_t group, per_claim;
     uint32_t n_groups;
-    // adjoint screening: frozen bunch counts, list of (step, bunch) pairs
+    // adjoint screening: frozen bunch counts (NULL: this launch's, written to
+    // y_nb), list of (step, bunch) pairs
     // that land within the read-out radius of a telescope centre
     const int32_t *nb_frozen;
     uint64_t *list;
@@ -233,21 +234,25 @@ struct KParams {
 struct AdjParams {
     KParams k;
     const uint64_t *list;
-    int64_t n_list;
+    const unsigned long long *count;      // listed bunches (device), list_cap entries
+    int64_t list_cap;
     const int32_t *nb;
     double sigma, inv_2s2, norm, rcut2;
+    float reach;                   // 6 sigma and the rounding of an FP32 difference
     double *S, *U;                 // [n_tel] read-out sums
     const double *gD, *gT;         // [n_tel] upstream gradients
     double *grad_atm;              // [15]: a_0..a_4, b_0..b_4, c_0..c_4
     double *grad_tracks;           // [6][n]: x0, y0, z0, ux, uy, uz
     const double *sens;            // [H][Z][20] table sensitivities
-    double hb[6], b[5], c[5];
+    double hb[6], c[5], inv_b[5], inv_c[5];
     int layer0;                    // layer of h = 0 (rho(0))
     double dh_fine;
-    int ko;                        // fine-table position of h_obs
-    double fo;
+    double dob[10];                // d eta(h_obs) / d p
 };
-cudaError_t adjoint_pairs(bool fp32, int mode, const AdjParams &A, void *stream);
+cudaError_t adjoint_pairs(bool fp32, int mode, const AdjParams &A, int num_sms, void *stream);
+// D_k = S_k, Tbar_k = U_k / S_k (either may be NULL)
+cudaError_t readout_values(const double *S, const double *U, double *D, double *T, int n_tel,
+                           void *stream);
 
 // Fill KParams::f from the double fields.
 void fill_float_constants(KParams &p);
