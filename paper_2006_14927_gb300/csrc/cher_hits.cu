@@ -304,6 +304,7 @@ struct alignas(16) WarpSmem : Spectra<R, DS>, SecRange<TR> {
     int nb[kCap + 1];             // bunches of each place
     int off[kCap + 33];           // first piece (kPer bunches) of each place, the
                                   // total, no more
+    unsigned long long n_emit, n_bunch;   // emitting steps and their bunches
     unsigned drop[6];             // bunches dropped, by status; [0]: invalid steps
 };
 
@@ -334,7 +335,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
     Consts<R> c;
     R np1o;
     make_consts<R>(p, c, np1o);
-    unsigned st_emit = 0, st_bunch = 0, st_hits = 0, st_over = 0;
+    if (lane == 0) W.n_emit = W.n_bunch = 0ull;
+    unsigned st_hits = 0, st_over = 0;
 
     // Groups of p.group steps, p.per_claim of them at a time: the first
     // claim is the warp's own number, the others come from the counter, one
@@ -419,8 +421,6 @@ __device__ __forceinline__ void hits(const KParams &p) {
                     if constexpr (MODE == MODE_HITS) {
                         if (p.prof && y.nb > 0) profile_call<R>(p, i, static_cast<R>(y.N));
                     }
-                    st_emit += y.nb > 0;
-                    st_bunch += y.nb;
                     if (!y.valid) atomicAdd(&W.drop[0], 1u);
                 }
                 if (!open && y.nb > 0) {
@@ -447,7 +447,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
                     }
                     kind = ring_setup<MODE, DS>(p, __double2float_rn(__ldg(p.x0 + i)),
                                                 __double2float_rn(__ldg(p.y0 + i)),
-                                                d2f_rn(z0) - p.f.h_obs, d2f_rn(len), ux, uy, uzf,
+                                                __double2float_rn(z0) - p.f.h_obs,
+                                                __double2float_rn(len), ux, uy, uzf,
                                                 eta, s_lo, s_hi,
                                                 *reinterpret_cast<Ring *>(&W.seg[cnt + lane]), B);
                 }
@@ -460,6 +461,14 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 }
             }
             const int nb = open ? 0 : y.nb;
+            if constexpr (MODE == MODE_HITS) {
+                const unsigned emit = __popc(__ballot_sync(kFull, nb > 0));
+                const unsigned sum = __reduce_add_sync(kFull, static_cast<unsigned>(nb));
+                if (lane == 0) {
+                    W.n_emit += emit;
+                    W.n_bunch += sum;
+                }
+            }
 
             // the telescopes near each lane's ring, then the pairs' sectors
             // (the places past cnt are free: their room holds the rings, and
@@ -724,12 +733,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
     if (MODE == MODE_HITS && S) {
         if (blockIdx.x == 0 && tid == 0)
             atomicAdd(S + CHER_STAT_STEPS, static_cast<unsigned long long>(p.n));
-        flush_stat(S, CHER_STAT_EMITTING, st_emit);
-        flush_stat(S, CHER_STAT_BUNCHES, st_bunch);
         __syncwarp();
-        const unsigned drop = lane >= ST_UPWARD && lane <= ST_ABSORBED ? W.drop[lane] : 0u;
-        if (lane == 0 && W.drop[0])
-            atomicAdd(S + CHER_STAT_INVALID, static_cast<unsigned long long>(W.drop[0]));
+        unsigned drop = lane >= ST_UPWARD && lane <= ST_ABSORBED ? W.drop[lane] : 0u;
         if (drop) {
             const int idx = lane == ST_UPWARD  ? CHER_STAT_UPWARD
                             : lane == ST_BELOW ? CHER_STAT_BELOW_OBS
@@ -738,9 +743,16 @@ __device__ __forceinline__ void hits(const KParams &p) {
                                                : CHER_STAT_ABSORBED;
             atomicAdd(S + idx, static_cast<unsigned long long>(drop));
         }
-        // reached the ground = generated - dropped (a per-thread partial may
-        // be negative; the sum modulo 2^64 is exact)
-        flush_stat_signed(S, CHER_STAT_GROUND, static_cast<int>(st_bunch) - static_cast<int>(drop));
+        drop = __reduce_add_sync(kFull, drop);
+        if (lane == 0) {
+            if (W.drop[0]) atomicAdd(S + CHER_STAT_INVALID, static_cast<unsigned long long>(W.drop[0]));
+            if (W.n_emit) {
+                atomicAdd(S + CHER_STAT_EMITTING, W.n_emit);
+                atomicAdd(S + CHER_STAT_BUNCHES, W.n_bunch);
+                // reached the ground = generated - dropped
+                atomicAdd(S + CHER_STAT_GROUND, W.n_bunch - drop);
+            }
+        }
         flush_stat(S, CHER_STAT_HITS, st_hits);
         flush_stat(S, CHER_STAT_OVERFLOW, st_over);
     }

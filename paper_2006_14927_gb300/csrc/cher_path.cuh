@@ -95,8 +95,9 @@ __device__ __forceinline__ bool screen_yield(const KParams &p, bool others_valid
         return true;
     y.valid = true;
     const float u = 5.9604645e-8f;                       // 2^-24
-    const float e = d2f_rn(ekin), L = d2f_rn(len);
-    const float z = d2f_rn(z0);
+    // (the FP64 pipe's conversions, idle otherwise: three instructions for sixty)
+    const float e = __double2float_rn(ekin), L = __double2float_rn(len);
+    const float z = __double2float_rn(z0);
     const float g = e * p.f.inv_me;
     const float gam = 1.0f + g, gam2 = gam * gam;
     float hm = z + (0.5f * L) * uz;
@@ -282,8 +283,9 @@ __device__ __forceinline__ bool screen_yield_disp(const KParams &p, bool others_
         return true;
     y.valid = true;
     const float u = 5.9604645e-8f;                       // 2^-24
-    const float e = d2f_rn(ekin), L = d2f_rn(len);
-    const float z = d2f_rn(z0);
+    // (the FP64 pipe's conversions, idle otherwise: three instructions for sixty)
+    const float e = __double2float_rn(ekin), L = __double2float_rn(len);
+    const float z = __double2float_rn(z0);
     const float g = e * p.f.inv_me;
     const float gam = 1.0f + g, gam2 = gam * gam;
     float hm = z + (0.5f * L) * uz;
