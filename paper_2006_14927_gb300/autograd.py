@@ -50,8 +50,8 @@ class _Readout(torch.autograd.Function):
                              fctx.sigma, fctx.nb)
         da, dp, dd = fctx.dtypes
         va, vp, vd = fctx.devices
-        grads = [gt[m].to(device=vp if m < 3 else vd, dtype=dp if m < 3 else dd)
-                 for m in range(6)]
+        # (one conversion for the three positions, one for the directions)
+        grads = [*gt[:3].to(device=vp, dtype=dp), *gt[3:].to(device=vd, dtype=dd)]
         return (ga.to(device=va, dtype=da), *grads, None, None, None, None, None, None, None,
                 None)
 

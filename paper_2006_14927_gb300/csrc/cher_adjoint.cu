@@ -124,6 +124,14 @@ __device__ __forceinline__ Dual<T> dsqrt(const Dual<T> &a) {
     return r;
 }
 
+// a launch constant in the path's precision (rounded on the host for FP32:
+// GB300 converts on its FP64 pipe)
+template <class T>
+__device__ __forceinline__ T lc(double d, float f) {
+    if constexpr (std::is_same<T, float>::value) return f;
+    else return d;
+}
+
 template <class T>
 __device__ __forceinline__ T tdir(const void *p, int64_t i) {
     return __ldg(static_cast<const T *>(p) + i);
@@ -136,8 +144,8 @@ __device__ __forceinline__ Dual<T> eta_dual(const KParams &p, const Dual<T> &h, 
                                             int &k_out, T &f_out) {
     T hc = h.v;
     if (hc < T(0)) hc = T(0);
-    if (hc > T(p.h_max)) hc = T(p.h_max);
-    const T x = hc * T(p.inv_dh);
+    if (hc > lc<T>(p.h_max, p.f.h_max)) hc = lc<T>(p.h_max, p.f.h_max);
+    const T x = hc * lc<T>(p.inv_dh, p.f.inv_dh);
     int k = static_cast<int>(x);
     k = k > p.n_fine - 2 ? p.n_fine - 2 : k;
     const T f = x - static_cast<T>(k);
@@ -149,8 +157,8 @@ __device__ __forceinline__ Dual<T> eta_dual(const KParams &p, const Dual<T> &h, 
         t0 = __ldg(p.eta64 + k);
         t1 = __ldg(p.eta64 + k + 1);
     }
-    const bool inside = h.v > T(0) && h.v < T(p.h_max);
-    const T slope = inside ? (t1 - t0) * T(p.inv_dh) : T(0);
+    const bool inside = h.v > T(0) && h.v < lc<T>(p.h_max, p.f.h_max);
+    const T slope = inside ? (t1 - t0) * lc<T>(p.inv_dh, p.f.inv_dh) : T(0);
     Dual<T> r = slope * h;
     r.v = t0 + f * (t1 - t0);
     r.d[channel] += T(1);
@@ -219,7 +227,7 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
     const T bg2 = g * (T(2) + g);
     const Dual<T> s2 = num / (bg2 * np1sq);
     if (!(s2.v > T(0)) || nb <= 0) return false;
-    const Dual<T> w = (static_cast<T>(p.K) * len / static_cast<T>(nb)) * s2;
+    const Dual<T> w = (lc<T>(p.K, p.f.K) * len / static_cast<T>(nb)) * s2;
     const T beta = sqrt(bg2) / gam;
     const Dual<T> cosc = cst<T>(T(1)) / (beta * np1);
     const Dual<T> sinc = dsqrt(s2);
@@ -259,10 +267,12 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
     const Dual<T> xe = x0 + fl * ux, ye = y0 + fl * uy, he = z0 + fl * uz;
     const T te = static_cast<T>(__ldg(p.t0 + i) - t_ref) + fl / (beta * T(kC));
     // rare conditions (a3)
-    if (!(pz.v < T(0)) || !(he.v >= T(p.h_obs)) || !(he.v <= T(p.h_max))) return false;
+    if (!(pz.v < T(0)) || !(he.v >= lc<T>(p.h_obs, p.f.h_obs)) ||
+        !(he.v <= lc<T>(p.h_max, p.f.h_max)))
+        return false;
     const Dual<T> eta_e = eta_dual<T>(p, he, C_ETA_E, o.ke, o.fe);
     o.he = static_cast<double>(he.v);
-    Dual<T> eta_o = cst<T>(static_cast<T>(p.eta_obs));
+    Dual<T> eta_o = cst<T>(lc<T>(p.eta_obs, p.f.eta_o));
     eta_o.d[C_ETA_O] = T(1);
     const Dual<T> se2 = px * px + py * py;
     if (!(se2.v > T(0))) return false;
@@ -270,16 +280,16 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
     const Dual<T> rat = (T(1) + eta_e) / (T(1) + eta_o);
     const Dual<T> sin_obs = sin_em * rat;
     const Dual<T> q = sin_obs * sin_obs;
-    if (!(q.v <= static_cast<T>(p.q_max))) return false;
+    if (!(q.v <= lc<T>(p.q_max, p.f.q_max))) return false;
     const Dual<T> cos_obs = dsqrt(cst<T>(T(1)) - q);
-    const Dual<T> dH = he - cst<T>(static_cast<T>(p.h_obs));
+    const Dual<T> dH = he - cst<T>(lc<T>(p.h_obs, p.f.h_obs));
     // table cell: value, slopes along dH and q, plus the table channels
-    const T fj = dH.v * static_cast<T>(p.inv_dht);
+    const T fj = dH.v * lc<T>(p.inv_dht, p.f.inv_dht);
     int jj = static_cast<int>(fj);
     jj = jj > p.H - 2 ? p.H - 2 : jj;
     jj = jj < 0 ? 0 : jj;
     const T a = fj - static_cast<T>(jj);
-    const T fk = q.v * static_cast<T>(p.inv_dq);
+    const T fk = q.v * lc<T>(p.inv_dq, p.f.inv_dq);
     int kk = static_cast<int>(fk);
     kk = kk > p.Z - 2 ? p.Z - 2 : kk;
     kk = kk < 0 ? 0 : kk;
@@ -305,8 +315,8 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
     }
     auto cell = [&](T v00, T v01, T v10, T v11, int channel) {
         const T v0 = v00 + a * (v10 - v00), v1 = v01 + a * (v11 - v01);
-        const T dvdh = ((T(1) - b) * (v10 - v00) + b * (v11 - v01)) * static_cast<T>(p.inv_dht);
-        const T dvdq = ((T(1) - a) * (v01 - v00) + a * (v11 - v10)) * static_cast<T>(p.inv_dq);
+        const T dvdh = ((T(1) - b) * (v10 - v00) + b * (v11 - v01)) * lc<T>(p.inv_dht, p.f.inv_dht);
+        const T dvdq = ((T(1) - a) * (v01 - v00) + a * (v11 - v10)) * lc<T>(p.inv_dq, p.f.inv_dq);
         Dual<T> r = dvdh * dH + dvdq * q;
         r.v = v0 + b * (v1 - v0);
         r.d[channel] += T(1);
@@ -332,49 +342,70 @@ __device__ bool bunch_dual(const AdjParams &A, int64_t i, int j, BunchDual<T> &o
     return true;
 }
 
-// Sums that many pairs add to the same few addresses (S_k, U_k per
-// telescope; the ten atmosphere gradients) are combined per CTA in shared
-// memory first, then added to global memory once per CTA: the pairs of a
-// shower crowd around a handful of telescopes.
-constexpr int kSmemTel = 512;     // telescopes whose S, U are combined in smem
+// The ten atmosphere gradients, to which every pair adds, are formed by the
+// warp with shuffles and kept per CTA in shared memory, which one lane adds to
+// (a CTA is one warp); S_k and U_k, per telescope, go out as FP64 reductions
+// to L2.  (FP64 atomics on shared memory are compare-and-swap loops: a warp
+// whose lanes all add to one address took 17 turns of the FP64 pipe per sum.)
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
 
 // One warp per CTA: a list of some thousand bunches is a long chain of FP64
 // work per thread (GB300: 2 FP64 lanes per SM and clock), so it is spread over
-// as many SMs as it has warps.  On the 300 GeV read-out (5e3 bunches listed):
-// FP32 recomputation, value pass 37.5 -> PAIRS0 us and gradient pass 120 ->
-// PAIRS1 us against CTAs of 128.
+// as many SMs as it has warps.  On the 300 GeV read-out (1e5 steps), FP32
+// recomputation: value pass 37.5 -> PAIRS0 us, gradient pass 120 -> PAIRS1 us
+// against CTAs of 128 with shared-memory atomics.
 constexpr int kPairBlock = 32;
 
 template <class T, int MODE>
 __global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
-    __shared__ double s_sum[MODE == 0 ? 2 * kSmemTel : 10];
-    const int n_tel = A.k.n_tel;
-    const bool smem_su = MODE == 0 && n_tel <= kSmemTel;
-    const int n_red = MODE == 0 ? (smem_su ? 2 * n_tel : 0) : 10;
-    for (int q = threadIdx.x; q < n_red; q += blockDim.x) s_sum[q] = 0.0;
-    __syncthreads();
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    __shared__ double s_sum[10];
+    const int n_tel = A.k.n_tel, lane = threadIdx.x;
     const unsigned long long listed = *A.count;
     const int64_t n_list = static_cast<int64_t>(
         listed < static_cast<unsigned long long>(A.list_cap) ? listed : A.list_cap);
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n_list;
-         e += stride) {
-        const uint64_t ent = A.list[e];
-        const int64_t i = static_cast<int64_t>(ent >> 32);
-        const int j = static_cast<int>(ent & 0xffffffffu);
+    if (static_cast<int64_t>(blockIdx.x) * kPairBlock >= n_list) return;
+    if (MODE == 1 && lane < 10) s_sum[lane] = 0.0;
+    __syncwarp();
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * kPairBlock;
+    for (int64_t e0 = static_cast<int64_t>(blockIdx.x) * kPairBlock; e0 < n_list; e0 += stride) {
+        const int64_t e = e0 + lane;
         BunchDual<T> o;
-        if (!bunch_dual<T>(A, i, j, o)) continue;
-        const double X = o.X.v, Y = o.Y.v, t = o.t.v, w = o.w.v;
+        int64_t i = 0;
+        bool live = e < n_list;
+        if (live) {
+            const uint64_t ent = A.list[e];
+            i = static_cast<int64_t>(ent >> 32);
+            live = bunch_dual<T>(A, i, static_cast<int>(ent & 0xffffffffu), o);
+        }
+        double X = 0, Y = 0, t = 0, w = 0;
+        float Xf = 0.0f, Yf = 0.0f;
+        if (live) {
+            X = o.X.v;
+            Y = o.Y.v;
+            t = o.t.v;
+            w = o.w.v;
+            Xf = static_cast<float>(o.X.v);
+            Yf = static_cast<float>(o.Y.v);
+        }
         double gX = 0, gY = 0, gt = 0, gw = 0;
         bool any = false;
-        const float Xf = static_cast<float>(o.X.v), Yf = static_cast<float>(o.Y.v);
-        for (int k = 0; k < A.k.n_tel; ++k) {
-            // most telescopes are out of reach: seen in FP32, with room for
-            // its rounding
-            const float4 C = __ldg(A.k.cull.tel + k);
-            if (!(fabsf(Xf - C.x) < A.reach && fabsf(Yf - C.y) < A.reach)) continue;
+        // Most telescopes are out of reach, which is seen in FP32 (with room
+        // for its rounding).  Every lane looks for its own next one first, so
+        // that the lanes' FP64 work on theirs runs together.
+        for (int k = live ? 0 : n_tel;; ++k) {
+            for (; k < n_tel; ++k) {
+                const float4 C = __ldg(A.k.cull.tel + k);
+                if (fabsf(Xf - C.x) < A.reach && fabsf(Yf - C.y) < A.reach) break;
+            }
+            if (!__any_sync(kFull, k < n_tel)) break;
+            if (k >= n_tel) continue;
             double tx, ty;
             if constexpr (std::is_same<T, float>::value) {
+                const float4 C = __ldg(A.k.cull.tel + k);
                 tx = C.x;
                 ty = C.y;
             } else {
@@ -387,13 +418,8 @@ __global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
             if (!(r2 < A.rcut2)) continue;
             const double G = A.norm * exp(-r2 * A.inv_2s2);
             if constexpr (MODE == 0) {
-                if (smem_su) {
-                    atomicAdd(s_sum + k, w * G);
-                    atomicAdd(s_sum + n_tel + k, w * G * t);
-                } else {
-                    atomicAdd(A.S + k, w * G);
-                    atomicAdd(A.U + k, w * G * t);
-                }
+                atomicAdd(A.S + k, w * G);
+                atomicAdd(A.U + k, w * G * t);
             } else {
                 const double S = __ldg(A.S + k), U = __ldg(A.U + k);
                 double dLdS = __ldg(A.gD + k), dLdU = 0.0;
@@ -412,44 +438,48 @@ __global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
             }
         }
         if constexpr (MODE == 1) {
-            if (!any) continue;
-            double gl[NT];
+            if (!__any_sync(kFull, any)) continue;
+            double gl[NT], dm[10], de[10], tab[20];
+            if (any) {
 #pragma unroll
-            for (int c = 0; c < NT; ++c)
-                gl[c] = gX * static_cast<double>(o.X.d[c]) + gY * static_cast<double>(o.Y.d[c]) +
-                        gt * static_cast<double>(o.t.d[c]) + gw * static_cast<double>(o.w.d[c]);
-            for (int m = 0; m < 6; ++m) atomicAdd(A.grad_tracks + m * A.k.n + i, gl[m]);
-            // atmosphere: the five channels through their sensitivities
-            double dm[10], de[10];
-            eta_sens(A, o.km, static_cast<double>(o.fm), dm);
-            eta_sens(A, o.ke, static_cast<double>(o.fe), de);
-            const double *s00 = A.sens + (static_cast<size_t>(o.jj) * A.k.Z + o.kk) * 20;
-            const double *s01 = s00 + 20;
-            const double *s10 = s00 + static_cast<size_t>(A.k.Z) * 20;
-            const double *s11 = s10 + 20;
-            const double aa = o.a, bb = o.b;
-            for (int q = 0; q < 10; ++q) {
-                double tab[2];
-                for (int m = 0; m < 2; ++m) {
-                    const int idx = m * 10 + q;
-                    const double v0 = __ldg(s00 + idx) + aa * (__ldg(s10 + idx) - __ldg(s00 + idx));
-                    const double v1 = __ldg(s01 + idx) + aa * (__ldg(s11 + idx) - __ldg(s01 + idx));
-                    tab[m] = v0 + bb * (v1 - v0);
+                for (int c = 0; c < NT; ++c)
+                    gl[c] = gX * static_cast<double>(o.X.d[c]) + gY * static_cast<double>(o.Y.d[c]) +
+                            gt * static_cast<double>(o.t.d[c]) + gw * static_cast<double>(o.w.d[c]);
+                for (int m = 0; m < 6; ++m) atomicAdd(A.grad_tracks + m * A.k.n + i, gl[m]);
+                // atmosphere: the five channels through their sensitivities
+                eta_sens(A, o.km, static_cast<double>(o.fm), dm);
+                eta_sens(A, o.ke, static_cast<double>(o.fe), de);
+                // (a node's 20 values are 160 bytes: 16-byte loads)
+                const double2 *s00 = reinterpret_cast<const double2 *>(
+                    A.sens + (static_cast<size_t>(o.jj) * A.k.Z + o.kk) * 20);
+                const double2 *s01 = s00 + 10;
+                const double2 *s10 = s00 + static_cast<size_t>(A.k.Z) * 10;
+                const double2 *s11 = s10 + 10;
+                const double aa = o.a, bb = o.b;
+#pragma unroll
+                for (int idx = 0; idx < 10; ++idx) {
+                    const double2 p00 = __ldg(s00 + idx), p01 = __ldg(s01 + idx);
+                    const double2 p10 = __ldg(s10 + idx), p11 = __ldg(s11 + idx);
+                    const double x0 = p00.x + aa * (p10.x - p00.x), x1 = p01.x + aa * (p11.x - p01.x);
+                    const double y0 = p00.y + aa * (p10.y - p00.y), y1 = p01.y + aa * (p11.y - p01.y);
+                    tab[2 * idx] = x0 + bb * (x1 - x0);
+                    tab[2 * idx + 1] = y0 + bb * (y1 - y0);
                 }
-                const double gp = gl[C_ETA_M] * dm[q] + gl[C_ETA_E] * de[q] +
-                                  gl[C_ETA_O] * A.dob[q] + gl[C_AX] * tab[0] + gl[C_AL] * tab[1];
-                atomicAdd(s_sum + q, gp);            // b_i at 5 + i, c_i at 10 + i
+            }
+#pragma unroll
+            for (int q = 0; q < 10; ++q) {
+                double gp = 0.0;
+                if (any)
+                    gp = gl[C_ETA_M] * dm[q] + gl[C_ETA_E] * de[q] + gl[C_ETA_O] * A.dob[q] +
+                         gl[C_AX] * tab[q] + gl[C_AL] * tab[10 + q];
+                gp = warp_sum(gp);
+                if (lane == 0) s_sum[q] += gp;       // b_i at 5 + i, c_i at 10 + i
             }
         }
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < n_red; q += blockDim.x) {
-        const double v = s_sum[q];
-        if (v == 0.0) continue;
-        if constexpr (MODE == 0)
-            atomicAdd(q < n_tel ? A.S + q : A.U + (q - n_tel), v);
-        else
-            atomicAdd(A.grad_atm + 5 + q, v);
+    if constexpr (MODE == 1) {
+        __syncwarp();
+        if (lane < 10 && s_sum[lane] != 0.0) atomicAdd(A.grad_atm + 5 + lane, s_sum[lane]);
     }
 }
 

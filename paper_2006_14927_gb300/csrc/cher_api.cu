@@ -823,7 +823,8 @@ cher_status cher_generate_steps(cher_ctx *c, const cher_shower *sh, int32_t n_sh
         return CHER_EINVAL;
     std::vector<cher::GenShower> G(n_showers);
     std::vector<int64_t> first(n_showers + 1, 0);
-    std::vector<float> cdf(static_cast<size_t>(n_showers) * kCdf);
+    constexpr int kRow = kCdf + cher::kGuideWords;
+    std::vector<float> cdf(static_cast<size_t>(n_showers) * kRow);
     std::vector<double> t_ref(n_showers), row;
     for (int s = 0; s < n_showers; ++s) {
         const cher_shower &S = sh[s];
@@ -861,9 +862,18 @@ cher_status cher_generate_steps(cher_ctx *c, const cher_shower *sh, int32_t n_sh
             if (c->cdf_cache.size() >= 4096) c->cdf_cache.clear();
             cher::greisen_cdf_host(std::log(S.e0_mev / kEc), t_g, kCdf, row);
             std::vector<float> rf(row.begin(), row.end());
+            // the guide behind the nodes: the last node at or below k / kGuide
+            rf.resize(kRow, 0.0f);
+            std::vector<uint16_t> guide(2 * cher::kGuideWords, 0);
+            int a = 0;
+            for (int k = 0; k <= cher::kGuide; ++k) {
+                while (a < kCdf - 2 && rf[a + 1] <= static_cast<float>(k) / cher::kGuide) ++a;
+                guide[k] = static_cast<uint16_t>(a);
+            }
+            std::memcpy(rf.data() + kCdf, guide.data(), sizeof(float) * cher::kGuideWords);
             it = c->cdf_cache.emplace(key, std::move(rf)).first;
         }
-        std::copy(it->second.begin(), it->second.end(), cdf.begin() + static_cast<size_t>(s) * kCdf);
+        std::copy(it->second.begin(), it->second.end(), cdf.begin() + static_cast<size_t>(s) * kRow);
     }
     // one scratch block: shower constants | offsets | tables, staged in pinned
     // host memory (with t_ref after it) and uploaded in one asynchronous copy

@@ -39,23 +39,43 @@ __device__ __forceinline__ float u01_full(uint32_t x) {
     return __uint2float_rn(x) * 2.3283064365386963e-10f + 1.1641532182693481e-10f;
 }
 
-__global__ void k_generate_steps(const GenParams g) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        // the shower of step i: the last first-index <= i
-        int lo = 0, hi = g.n_showers;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(g.first + mid) <= i) lo = mid; else hi = mid;
+// A CTA takes a contiguous run of the steps, so that a thread meets a new
+// shower rarely: the first is searched for, the next ones are the following
+// ones, and the shower's constants stay in registers in between.  The depth's
+// CDF node comes from a guide, the node below each of kGuide + 1 equally
+// spaced deviates, and a bisection between two of its entries (one or two
+// steps in the bulk against ten over the whole row).
+__global__ void __launch_bounds__(256) k_generate_steps(const GenParams g) {
+    const int64_t chunk = (g.n + gridDim.x - 1) / gridDim.x;
+    const int64_t i0 = blockIdx.x * chunk, i1 = i0 + chunk < g.n ? i0 + chunk : g.n;
+    int lo = -1;
+    int64_t lo_end = 0;
+    GenShower S;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+        if (lo < 0 || i >= lo_end) {
+            // the shower of step i: the last first-index <= i
+            if (lo < 0) {
+                int hi = g.n_showers;
+                lo = 0;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (__ldg(g.first + mid) <= i) lo = mid; else hi = mid;
+                }
+            } else {
+                while (lo + 1 < g.n_showers && __ldg(g.first + lo + 1) <= i) ++lo;
+            }
+            lo_end = __ldg(g.first + lo + 1);
+            S = g.showers[lo];
         }
-        const GenShower S = g.showers[lo];
         const uint32_t c0 = static_cast<uint32_t>(i), c1 = static_cast<uint32_t>(i >> 32);
         const uint4 w0 = dev::philox4x32_10(make_uint4(c0, c1, 0u, 1u), g.key0, g.key1);
         const uint4 w1 = dev::philox4x32_10(make_uint4(c0, c1, 1u, 1u), g.key0, g.key1);
         // depth from the tabulated CDF of this shower
-        const float *F = g.cdf + static_cast<int64_t>(lo) * g.n_cdf;
+        const float *F = g.cdf + static_cast<int64_t>(lo) * (g.n_cdf + kGuideWords);
         const float u0 = u01_full(w0.x);
-        int a = 0, b = g.n_cdf - 1;
+        const uint16_t *G = reinterpret_cast<const uint16_t *>(F + g.n_cdf) +
+                            min(static_cast<int>(u0 * kGuide), kGuide - 1);
+        int a = __ldg(G), b = min(__ldg(G + 1) + 1, g.n_cdf - 1);
         while (b - a > 1) {
             const int mid = (a + b) >> 1;
             if (__ldg(F + mid) <= u0) a = mid; else b = mid;
@@ -103,7 +123,7 @@ __global__ void k_generate_steps(const GenParams g) {
 
 cudaError_t generate_steps(const GenParams &g, int num_sms, void *stream) {
     if (g.n <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((g.n + 255) / 256, int64_t(num_sms) * 16);
+    const int64_t blocks = std::min<int64_t>((g.n + 255) / 256, int64_t(num_sms) * 8);
     k_generate_steps<<<static_cast<int>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(g);
     return cudaGetLastError();
 }

@@ -295,17 +295,21 @@ size_t hits_smem_bytes(bool fp32, int mode, int block);
 // Launchers (cher_kernels.cu).  fp32 selects CHER_FP32_BULK.
 size_t kernel_smem_bytes(bool fp32, int block, int mode, const KParams &p);
 // Device step generator (cher_generator.cu): per-shower constants in float.
-struct GenShower {
+// A row of the CDF: n_cdf nodes, then the guide (kGuide + 1 16-bit indices:
+// the last node whose value is at most k / kGuide).
+constexpr int kGuide = 256, kGuideWords = 132;
+struct alignas(16) GenShower {
     float ax, ay, az;            // axis (downward)
     float b1x, b1y, b1z, b2x, b2y, b2z;   // transverse basis
     float cz, x0cz;              // cos zenith, X0 cos zenith (g/cm^2)
     float core_x, core_y, s_ref, dt;      // s_ref: m; dt: CDF node spacing
+    float pad;
 };
 struct GenParams {
     const GenShower *showers;
     const int64_t *first;        // [n_showers + 1] first global step of each shower
     int32_t n_showers, n_cdf;
-    const float *cdf;            // [n_showers][n_cdf]
+    const float *cdf;            // [n_showers][n_cdf + kGuideWords]
     uint32_t key0, key1;
     float h_obs;
     int64_t n;
