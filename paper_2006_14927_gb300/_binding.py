@@ -423,8 +423,8 @@ class Context:
         torch = _torch()
         n = int(dev_tracks["x0"].numel())
         dev = dev_tracks["x0"].device
-        nb = torch.zeros(n, dtype=torch.int32, device=dev)
-        w = torch.zeros(n, dtype=torch.float64, device=dev)
+        nb = torch.empty(n, dtype=torch.int32, device=dev)              # (all written)
+        w = torch.empty(n, dtype=torch.float64, device=dev)
         t = self.tracks_struct(dev_tracks)
         _check(lib().cher_segment_yield(self._h, ctypes.byref(t), int(precision), nb.data_ptr(),
                                         w.data_ptr(), ctypes.c_void_p(_stream_ptr(stream))),

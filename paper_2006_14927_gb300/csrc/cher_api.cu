@@ -875,13 +875,12 @@ cher_status cher_generate_steps(cher_ctx *c, const cher_shower *sh, int32_t n_sh
         }
         std::copy(it->second.begin(), it->second.end(), cdf.begin() + static_cast<size_t>(s) * kRow);
     }
-    // one scratch block: shower constants | offsets | tables, staged in pinned
-    // host memory (with t_ref after it) and uploaded in one asynchronous copy
+    // one scratch block: shower constants | offsets | tables | reference
+    // times, staged in pinned host memory and uploaded in one asynchronous copy
     const size_t o_first = (sizeof(cher::GenShower) * n_showers + 15) & ~size_t(15);
     const size_t o_cdf = (o_first + sizeof(int64_t) * (n_showers + 1) + 15) & ~size_t(15);
-    const size_t bytes = o_cdf + sizeof(float) * cdf.size();
-    const size_t o_tref = (bytes + 15) & ~size_t(15);
-    const size_t staged = o_tref + sizeof(double) * n_showers;
+    const size_t o_tref = (o_cdf + sizeof(float) * cdf.size() + 15) & ~size_t(15);
+    const size_t bytes = o_tref + sizeof(double) * n_showers;
     cher_status r;
     if ((r = grow(&c->d_gen, c->gen_cap, static_cast<int64_t>(bytes))) != CHER_OK) return r;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -893,25 +892,23 @@ cher_status cher_generate_steps(cher_ctx *c, const cher_shower *sh, int32_t n_sh
     // the previous call's upload has read the staging before it is rewritten
     if (c->gen_ev_pending && cudaEventSynchronize(c->gen_ev) != cudaSuccess) return CHER_ECUDA;
     c->gen_ev_pending = false;
-    if (static_cast<int64_t>(staged) > c->h_gen_cap) {
+    if (static_cast<int64_t>(bytes) > c->h_gen_cap) {
         cudaFreeHost(c->h_gen);
         c->h_gen = nullptr;
         c->h_gen_cap = 0;
         void *h = nullptr;
-        if (cudaHostAlloc(&h, staged, cudaHostAllocDefault) != cudaSuccess) {
+        if (cudaHostAlloc(&h, bytes, cudaHostAllocDefault) != cudaSuccess) {
             cudaGetLastError();
             return CHER_ENOMEM;
         }
         c->h_gen = static_cast<unsigned char *>(h);
-        c->h_gen_cap = static_cast<int64_t>(staged);
+        c->h_gen_cap = static_cast<int64_t>(bytes);
     }
     std::memcpy(c->h_gen, G.data(), sizeof(cher::GenShower) * n_showers);
     std::memcpy(c->h_gen + o_first, first.data(), sizeof(int64_t) * (n_showers + 1));
     std::memcpy(c->h_gen + o_cdf, cdf.data(), sizeof(float) * cdf.size());
     std::memcpy(c->h_gen + o_tref, t_ref.data(), sizeof(double) * n_showers);
     if (cudaMemcpyAsync(c->d_gen, c->h_gen, bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(out->t_ref, c->h_gen + o_tref, sizeof(double) * n_showers,
-                        cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaEventRecord(c->gen_ev, st) != cudaSuccess)
         return CHER_ECUDA;
     c->gen_ev_pending = true;
@@ -930,6 +927,8 @@ cher_status cher_generate_steps(cher_ctx *c, const cher_shower *sh, int32_t n_sh
     g.ux = out->ux; g.uy = out->uy; g.uz = out->uz;
     g.dirs_fp32 = prec == CHER_FP32_BULK;
     g.shower = out->shower;
+    g.t_ref_in = reinterpret_cast<const double *>(c->d_gen + o_tref);
+    g.t_ref = out->t_ref;
     if (cher::generate_steps(g, c->num_sms, stream) != cudaSuccess) return CHER_ECUDA;
     return CHER_OK;
 }

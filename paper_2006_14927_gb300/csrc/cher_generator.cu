@@ -46,6 +46,9 @@ __device__ __forceinline__ float u01_full(uint32_t x) {
 // spaced deviates, and a bisection between two of its entries (one or two
 // steps in the bulk against ten over the whole row).
 __global__ void __launch_bounds__(256) k_generate_steps(const GenParams g) {
+    // the showers' reference times, to the caller's array
+    if (blockIdx.x == 0)
+        for (int s = threadIdx.x; s < g.n_showers; s += blockDim.x) g.t_ref[s] = g.t_ref_in[s];
     const int64_t chunk = (g.n + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = blockIdx.x * chunk, i1 = i0 + chunk < g.n ? i0 + chunk : g.n;
     int lo = -1;
@@ -122,8 +125,7 @@ __global__ void __launch_bounds__(256) k_generate_steps(const GenParams g) {
 }  // namespace
 
 cudaError_t generate_steps(const GenParams &g, int num_sms, void *stream) {
-    if (g.n <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((g.n + 255) / 256, int64_t(num_sms) * 8);
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((g.n + 255) / 256, int64_t(num_sms) * 8));
     k_generate_steps<<<static_cast<int>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(g);
     return cudaGetLastError();
 }

@@ -317,6 +317,8 @@ struct GenParams {
     void *ux, *uy, *uz;
     bool dirs_fp32;
     uint32_t *shower;
+    const double *t_ref_in;      // [n_showers]
+    double *t_ref;
 };
 cudaError_t generate_steps(const GenParams &g, int num_sms, void *stream);
 // The Greisen profile's CDF on n_cdf uniform nodes of [0, t_g] (host, FP64).
