@@ -79,12 +79,16 @@ struct alignas(16) Ring {
 
 enum : int { REACH_NONE = 0, REACH_RING = 1, REACH_ALL = 2 };
 
+// What the first test of one telescope needs besides (32 bytes, behind the
+// Ring): the axis's ground point, the distance to it times the cone's sine,
+// rho <= R fac + c1; the slack of r_k^2 and the axis's arrival direction.
+struct alignas(16) Near {
+    float4 p;      // P (x, y), sm a_0, c1
+    float4 w;      // u' (x, y, z), E
+};
+
 struct Box {
     uint32_t bins;                // of the telescopes' centres: x0, x1 + 1, y0, y1 + 1
-    float Px, Py;                 // the axis's ground point
-    float wx, wy, wz;             // the axis's arrival direction
-    float sm, ra0, cm2;           // r_c = sm (D.u') + ra0, r_k^2 = cm2 (D^2 - (D.u')^2)
-    float fac, c1, E;             // first test: rho <= R fac + c1, slack of r_k^2
     float sec_lo, sec_hi;         // bounds of 1 / cos(theta_o) over the step's bunches
 };
 
@@ -94,7 +98,7 @@ struct Box {
 template <int MODE, bool DS>
 __device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, float dz0, float L,
                                           float ux, float uy, float uz, float eta, float sinc_lo,
-                                          float sinc_hi, Ring &G, Box &B) {
+                                          float sinc_hi, Ring &G, Near &N, Box &B) {
     const float su2 = ux * ux + uy * uy;
     // the step points down, is a unit vector, and its cone is narrow
     bool ok = (uz < 0.0f) & (fabsf(su2 + uz * uz - 1.0f) <= 4e-6f) & (sinc_hi <= 0.25f);
@@ -175,9 +179,8 @@ __device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, 
     const float ca = fabsf(e1y), sa = fabsf(e1x);        // the step's azimuth
     const float bwx = along * ca + across * sa + slack, bwy = along * sa + across * ca + slack;
     const float a0 = sec * dzm, t = rat * a0;
-    B.Px = X0 + t * ux;
-    B.Py = Y0 + t * uy;
-    const float bx = (B.Px - p.cull.x0) * p.cull.inv_bx, by = (B.Py - p.cull.y0) * p.cull.inv_by;
+    const float Px = X0 + t * ux, Py = Y0 + t * uy;
+    const float bx = (Px - p.cull.x0) * p.cull.inv_bx, by = (Py - p.cull.y0) * p.cull.inv_by;
     const int b0 = max(__float2int_rd(bx - bwx * p.cull.inv_bx), 0);
     const int b1 = min(__float2int_rd(bx + bwx * p.cull.inv_bx), kCullBins - 1);
     const int b2 = max(__float2int_rd(by - bwy * p.cull.inv_by), 0);
@@ -189,18 +192,12 @@ __device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, 
     // D = C - P: w.u' = a_0 + D.u' and |w|^2 - (w.u')^2 = D^2 - (D.u')^2; rho
     // at the largest distance in the box, and the rounding of the squares
     const float w_max = a0 + 1.42f * fmaxf(bwx, bwy) + half + p.cull.z_max;
-    B.wx = ux + dx;
-    B.wy = uy + dy;
-    B.wz = uz + dz;
-    B.sm = sm;
-    B.ra0 = sm * a0;
-    B.cm2 = 1.0f - sm * sm;
-    B.fac = fac;
-    B.c1 = mo * fac + 0.1f + (mw * fac + spread + 2.5f * bs * sinc_hi) * w_max;
-    B.E = 4e-6f * (bwx * bwx + bwy * bwy);
+    const float c1 = mo * fac + 0.1f + (mw * fac + spread + 2.5f * bs * sinc_hi) * w_max;
+    N.p = make_float4(Px, Py, sm * a0, c1);
+    N.w = make_float4(ux + dx, uy + dy, uz + dz, 4e-6f * (bwx * bwx + bwy * bwy));
     // a step well above every sphere: no line comes to one from behind or from
     // the side (the tests below take a = w.u' > 0 and far from the cone's side)
-    ok = ok & (dzm > p.cull.z_max + 2.5f * (r_max * fac + B.c1));
+    ok = ok & (dzm > p.cull.z_max + 2.5f * (r_max * fac + c1));
     return !ok ? REACH_ALL : (b0 <= b1 && b2 <= b3 ? REACH_RING : REACH_NONE);
 }
 
@@ -308,12 +305,43 @@ struct alignas(16) WarpSmem : Spectra<R, DS>, SecRange<TR> {
     unsigned drop[6];             // bunches dropped, by status; [0]: invalid steps
 };
 
-// Pair q (up to kNear x 32) of a group: the free places past cnt hold a Ring in
-// their first 64 bytes and pairs in the next 32.
-template <class W>
-__device__ __forceinline__ uint32_t &pair_slot(W &w, int cnt, int q) {
-    return reinterpret_cast<uint32_t *>(&w.seg[cnt + (q & 31)])[16 + (q >> 5)];
+// Word w of the telescopes in a box of bins.
+__device__ __forceinline__ uint32_t box_telescopes(const KParams &p, uint32_t bins, int w) {
+    const int nw = p.cull.words;
+    const uint32_t *X = p.cull.bins + w, *Y = X + (kCullBins + 1) * nw;
+    return __ldg(X + (bins >> 8 & 0xffu) * nw) & ~__ldg(X + (bins & 0xffu) * nw) &
+           __ldg(Y + (bins >> 24) * nw) & ~__ldg(Y + (bins >> 16 & 0xffu) * nw);
 }
+
+// inclusive prefix sum over the warp
+__device__ __forceinline__ int warp_scan(int v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// While a group is worked on, the places past cnt are free: place cnt + lane
+// holds the lane's Ring and Near, and its mask collects the sectors; the pairs
+// that pass the first test (two a lane at a time) are listed where the free
+// places' offsets will be.
+template <class W>
+__device__ __forceinline__ Ring *ring_at(W &w, int place) {
+    return reinterpret_cast<Ring *>(&w.seg[place]);
+}
+template <class W>
+__device__ __forceinline__ Near *near_at(W &w, int place) {
+    return reinterpret_cast<Near *>(reinterpret_cast<unsigned char *>(&w.seg[place]) + sizeof(Ring));
+}
+constexpr int kPairs = 64;
+template <class W>
+__device__ __forceinline__ uint32_t &pair_at(W &w, int q) {
+    return reinterpret_cast<uint32_t *>(w.off + kCap - 32)[q];
+}
+static_assert(sizeof(Ring) + sizeof(Near) <= sizeof(Seg<float>), "a free place holds both");
+static_assert(kCap - 32 + kPairs <= kCap + 33, "the pairs fit the free places' offsets");
 
 template <class R, int MODE, bool TR, int FB, bool DS>
 __device__ __forceinline__ void hits(const KParams &p) {
@@ -450,7 +478,7 @@ __device__ __forceinline__ void hits(const KParams &p) {
                                                 __double2float_rn(z0) - p.f.h_obs,
                                                 __double2float_rn(len), ux, uy, uzf,
                                                 eta, s_lo, s_hi,
-                                                *reinterpret_cast<Ring *>(&W.seg[cnt + lane]), B);
+                                                *ring_at(W, cnt + lane), *near_at(W, cnt + lane), B);
                 }
             }
             if constexpr (std::is_same<R, float>::value) {
@@ -470,66 +498,69 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 }
             }
 
-            // the telescopes near each lane's ring, then the pairs' sectors
-            // (the places past cnt are free: their room holds the rings, and
-            // their masks collect the sectors)
+            // the telescopes near each lane's ring (32 to a word, from the box
+            // by the bins' prefix masks), then the sectors of those pairs
 #pragma unroll
             for (int w = 0; w < kMaskWords; ++w) W.mask[cnt + lane][w] = 0u;
             int n_near = 0;
             if (kind == REACH_RING) {
-                // the box's telescopes, 32 to a word: prefix masks of the bins
-                const int nw = p.cull.words;
-                const uint32_t *X = p.cull.bins, *Y = X + (kCullBins + 1) * nw;
-                const uint32_t *X0 = X + (B.bins & 0xffu) * nw, *X1 = X + (B.bins >> 8 & 0xffu) * nw;
-                const uint32_t *Y0 = Y + (B.bins >> 16 & 0xffu) * nw, *Y1 = Y + (B.bins >> 24) * nw;
-                for (int w = 0; w < nw; ++w) {
-                    uint32_t cand = __ldg(X1 + w) & ~__ldg(X0 + w) & __ldg(Y1 + w) & ~__ldg(Y0 + w);
+                const Ring *G = ring_at(W, cnt + lane);
+                const Near *N = near_at(W, cnt + lane);
+                const float sm = G->a.w, fac = G->e.z, cm2 = 1.0f - sm * sm;
+                const float4 P = N->p, U = N->w;
+                for (int w = 0; w < p.cull.words; ++w) {
+                    uint32_t cand = box_telescopes(p, B.bins, w);
                     while (cand) {
                         const int m = w * 32 + __ffs(cand) - 1;
                         cand &= cand - 1u;
                         const float4 T = __ldg(p.cull.tel + dbg_index(p, m, p.n_tel, DBG_GRID));
-                        const float dx = T.x - B.Px, dy = T.y - B.Py;
+                        const float dx = T.x - P.x, dy = T.y - P.y;
                         const float dz = MODE == MODE_SCREEN ? 0.0f : T.z;
-                        const float dot = dx * B.wx + dy * B.wy + dz * B.wz;
-                        const float rk2 = B.cm2 * (dx * dx + dy * dy + dz * dz - dot * dot);
-                        const float rc = B.sm * dot + B.ra0;
-                        const float rho = (MODE == MODE_SCREEN ? p.cull.r_cut : T.w) * B.fac + B.c1;
+                        const float dot = dx * U.x + dy * U.y + dz * U.z;
+                        const float rk2 = cm2 * (dx * dx + dy * dy + dz * dz - dot * dot);
+                        const float rc = sm * dot + P.z;
+                        const float rho = (MODE == MODE_SCREEN ? p.cull.r_cut : T.w) * fac + P.w;
                         const float far = rc + rho, near = fmaxf(rc - rho, 0.0f);
-                        const bool in = (rk2 <= far * far + B.E) & (rk2 >= near * near - B.E);
+                        const bool in = (rk2 <= far * far + U.w) & (rk2 >= near * near - U.w);
                         if (in) W.near[n_near & (kNear - 1)][lane] = static_cast<uint16_t>(m);
                         n_near += in;
                     }
                 }
-                if (n_near > kNear) kind = REACH_ALL;
-            }
-            // the pairs, lane by lane into one list (in the rest of the places)
-            n_near = kind == REACH_RING ? n_near : 0;
-            int n_pairs = 0;
-            for (int k = 0;; ++k) {
-                const unsigned has = __ballot_sync(kFull, n_near > k);
-                if (has == 0u) break;
-                if (n_near > k) {
-                    const int q = n_pairs + __popc(has & below);
-                    pair_slot(W, cnt, q) = (static_cast<uint32_t>(lane) << 16) | W.near[k][lane];
-                }
-                n_pairs += __popc(has);
-            }
-            __syncwarp();
-            for (int q = lane; q < n_pairs; q += 32) {
-                const uint32_t e = pair_slot(W, cnt, q);
-                const int at = cnt + static_cast<int>(e >> 16);
-                const Ring H = *reinterpret_cast<const Ring *>(&W.seg[at]);
-                const int2 k = ring_sectors<MODE>(p, H, __ldg(p.cull.tel + (e & 0xffffu)));
-                // sectors k.x .. k.x + k.y - 1 around the circle, word by word
-                for (int s = k.x, n = k.y; n > 0;) {
-                    const int b = s & 31, m = min(32 - b, n);
-                    atomicOr(&W.mask[at][(s >> 5) & (kMaskWords - 1)],
-                             (m == 32 ? kFull : (1u << m) - 1u) << b);
-                    s += m;
-                    n -= m;
+                if (n_near > kNear) {
+                    kind = REACH_ALL;
+                    n_near = 0;
                 }
             }
             __syncwarp();
+            // two telescopes a lane at a time: one round of full lanes for the
+            // usual 19 - 30 pairs of a group
+            for (int k0 = 0; __any_sync(kFull, n_near > k0); k0 += 2) {
+                int n_pairs = 0;
+#pragma unroll
+                for (int k = k0; k < k0 + 2; ++k) {
+                    const unsigned has = __ballot_sync(kFull, n_near > k);
+                    if (n_near > k)
+                        pair_at(W, n_pairs + __popc(has & below)) =
+                            static_cast<uint32_t>(cnt + lane) << 16 | W.near[k][lane];
+                    n_pairs += __popc(has);
+                }
+                __syncwarp();
+                for (int q = lane; q < n_pairs; q += 32) {
+                    const uint32_t e = pair_at(W, q);
+                    const int at = static_cast<int>(e >> 16);
+                    const int2 sec = ring_sectors<MODE>(p, *ring_at(W, at),
+                                                        __ldg(p.cull.tel + (e & 0xffffu)));
+                    // sectors sec.x .. sec.x + sec.y - 1 around the circle, word by word
+                    for (int s = sec.x, n = sec.y; n > 0;) {
+                        const int b = s & 31, m = min(32 - b, n);
+                        atomicOr(&W.mask[at][(s >> 5) & (kMaskWords - 1)],
+                                 (m == 32 ? kFull : (1u << m) - 1u) << b);
+                        s += m;
+                        n -= m;
+                    }
+                }
+                __syncwarp();
+            }
             uint32_t mask[kMaskWords], any = 0u;
 #pragma unroll
             for (int w = 0; w < kMaskWords; ++w) {
@@ -540,12 +571,7 @@ __device__ __forceinline__ void hits(const KParams &p) {
             const bool keep = nb > 0 && (kDraw || any != 0u);
             const unsigned kept = __ballot_sync(kFull, keep);
             const int np = (nb + kPer - 1) / kPer;
-            int v = keep ? np : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(kFull, v, o);
-                if (lane >= o) v += t;
-            }
+            const int v = warp_scan(keep ? np : 0, lane);
             if (keep) {
                 const int s = dbg_index(p, cnt + __popc(kept & below), kCap, DBG_SMEM);
                 W.off[s] = tot + v - np;
@@ -759,9 +785,10 @@ __device__ __forceinline__ void hits(const KParams &p) {
 }
 
 // One instantiation for every block size: 64 registers in FP32 (1024 threads
-// per SM), 128 in FP64.
+// per SM), 128 in FP64.  With spectra (128-step blocks only) 72: seven CTAs per
+// SM without spills against eight with them, 144 -> 136 us at 3e5 steps.
 template <class R, int MODE, bool TR, int FB, bool DS>
-__global__ void __launch_bounds__(512, std::is_same<R, float>::value ? 2 : 1)
+__global__ void __launch_bounds__(DS ? 128 : 512, std::is_same<R, float>::value ? (DS ? 7 : 2) : 1)
     k_hits(const __grid_constant__ KParams p) {
     hits<R, MODE, TR, FB, DS>(p);
 }

@@ -598,15 +598,26 @@ void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
 }
 
 void table_slopes(const HostTables &T, double &per_q, double &per_h) {
-    per_q = per_h = 0.0;
-    for (int j = 0; j < T.H; ++j)
-        for (int k = 0; k < T.Z; ++k) {
-            const size_t a = static_cast<size_t>(j) * T.Z + k;
-            if (k + 1 < T.Z)
-                per_q = std::max(per_q, std::fabs(T.ax[a + 1] - T.ax[a]) * T.inv_dq);
+    // (rows shared out over threads: a 4000 x 256 table takes a few ms otherwise)
+    const int nthr = std::max(1, std::min(16, T.H / 64));
+    std::vector<double> mq(nthr, 0.0), mh(nthr, 0.0);
+    auto rows = [&](int t) {
+        double q = 0.0, h = 0.0;
+        for (int j = t * T.H / nthr; j < (t + 1) * T.H / nthr; ++j) {
+            const double *a = T.ax.data() + static_cast<size_t>(j) * T.Z;
+            for (int k = 0; k + 1 < T.Z; ++k) q = std::max(q, std::fabs(a[k + 1] - a[k]));
             if (j + 1 < T.H)
-                per_h = std::max(per_h, std::fabs(T.ax[a + T.Z] - T.ax[a]) * T.inv_dht);
+                for (int k = 0; k < T.Z; ++k) h = std::max(h, std::fabs(a[k + T.Z] - a[k]));
         }
+        mq[t] = q;
+        mh[t] = h;
+    };
+    std::vector<std::thread> pool;
+    for (int t = 1; t < nthr; ++t) pool.emplace_back(rows, t);
+    rows(0);
+    for (auto &th : pool) th.join();
+    per_q = *std::max_element(mq.begin(), mq.end()) * T.inv_dq;
+    per_h = *std::max_element(mh.begin(), mh.end()) * T.inv_dht;
 }
 
 // Greisen profile of a shower of y = ln(E0 / E_c), up to a constant factor,
