@@ -41,8 +41,7 @@ struct cher_ctx {
     double *d_cand64[2] = {nullptr, nullptr};
     // the hits kernel's bins of telescope centres and table slopes
     cher::HostBins CB;
-    uint32_t *d_cull_bins = nullptr;
-    float *d_cull_tel = nullptr;
+    float *d_cull = nullptr;              // the telescopes, then the bins' masks
     double cull_rmax = 0, cull_zmax = 0, ax_sq = 0, ax_sh = 0;
     // scratch: the persistent kernel's tile counter
     unsigned *d_scratch = nullptr;
@@ -114,10 +113,8 @@ void free_tables(cher_ctx *c) {
         c->d_cand32[g] = nullptr;
         c->d_cand64[g] = nullptr;
     }
-    cudaFree(c->d_cull_bins);
-    cudaFree(c->d_cull_tel);
-    c->d_cull_bins = nullptr;
-    c->d_cull_tel = nullptr;
+    cudaFree(c->d_cull);
+    c->d_cull = nullptr;
     c->d_eta64 = nullptr;
     c->d_eta32 = nullptr;
     c->d_tab64 = c->d_tab32 = nullptr;
@@ -333,8 +330,8 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
     p.cull.inv_by = static_cast<float>(c->CB.inv_by);
     p.cull.r_max = static_cast<float>(c->cull_rmax);
     p.cull.z_max = static_cast<float>(c->cull_zmax);
-    p.cull.bins = c->d_cull_bins;
-    p.cull.tel = reinterpret_cast<const float4 *>(c->d_cull_tel);
+    p.cull.tel = reinterpret_cast<const float4 *>(c->d_cull);
+    p.cull.bins = reinterpret_cast<const uint32_t *>(c->d_cull + 4 * c->tel.size());
     // the layered thickness, for the production profile
     for (int l = 0; l < 6; ++l) p.atm.hb[l] = c->atm.h_bound[l];
     for (int l = 0; l < 5; ++l) {
@@ -645,6 +642,9 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
         c->cull_rmax = std::max(c->cull_rmax, q.r * (1.0 + 1e-6));
         c->cull_zmax = std::max(c->cull_zmax, std::fabs(q.z) * (1.0 + 1e-6));
     }
+    const size_t n_masks = c->CB.masks.size();
+    ctel.resize(4 * nt + n_masks);
+    std::memcpy(ctel.data() + 4 * nt, c->CB.masks.data(), n_masks * sizeof(uint32_t));
     cher::table_slopes(c->T, c->ax_sq, c->ax_sh);
     cher_status r;
     double *d_tab64 = nullptr;
@@ -656,8 +656,7 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
         (r = upload(&d_tab32, t32.data(), t32.size())) != CHER_OK ||
         (r = upload(&d_tel64, tel64.data(), tel64.size())) != CHER_OK ||
         (r = upload(&d_tel32, tel32.data(), tel32.size())) != CHER_OK ||
-        (r = upload(&c->d_cull_bins, c->CB.masks.data(), c->CB.masks.size())) != CHER_OK ||
-        (r = upload(&c->d_cull_tel, ctel.data(), ctel.size())) != CHER_OK ||
+        (r = upload(&c->d_cull, ctel.data(), ctel.size())) != CHER_OK ||
         (r = upload_grid(c, 0)) != CHER_OK || (r = upload_grid(c, 1)) != CHER_OK) {
         c->d_tab64 = d_tab64;
         c->d_tab32 = d_tab32;

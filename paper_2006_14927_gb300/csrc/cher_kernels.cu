@@ -1,5 +1,7 @@
-// cher_kernels.cu -- the hot path (steps a1-a5) as one fused kernel per tile
-// of track steps, in FP64 and in FP32-bulk precision.
+// cher_kernels.cu -- every bunch of a tile of track steps, in FP64 and in
+// FP32-bulk precision: the yields, the trace and, in a curved atmosphere, the
+// crossings (steps a1-a5; in flat layers cher_hits.cu forms those without
+// propagating every bunch).
 //
 // A CTA owns a tile of `BLOCK` consecutive steps:
 //   phase A  one thread per step: Cherenkov yield (CERENK, paper section
@@ -18,8 +20,8 @@
 //            hoisting of Algorithm 3), the ground point and arrival time
 //            (RAYBND, Appendix B listing), candidate spheres from the ground
 //            grid, and warp-aggregated compaction of the crossings (TELOUT;
-//            the hits kernels queue their crossings per warp and record
-//            them 32 at a time, see flush_ring).
+//            the curved hits kernels queue their crossings per warp and
+//            record them 32 at a time, see flush_ring).
 // In the persistent variant CTAs pull tiles from an atomic queue, so showers
 // of very uneven size share one launch (the paper's independent-shower
 // parallelism, section 2, inside one GPU).
@@ -36,8 +38,8 @@
 namespace cher {
 namespace {
 
-// The hits kernels record their crossings from a per-warp queue instead of
-// in the window where they are found.  About 1-2 % of bunches cross a
+// The curved hits kernels record their crossings from a per-warp queue instead
+// of in the window where they are found.  About 1-2 % of bunches cross a
 // sphere, so a window usually holds none or one, and recording it there
 // keeps 31 of 32 lanes idle through the record's ~70 instructions.  The
 // window queues each (bunch, candidate) pair as 8 bytes (step in tile and
@@ -46,9 +48,9 @@ namespace {
 // are still in shared memory, each lane takes one pair, computes its bunch
 // again (the same function on the same inputs, so the same values) and
 // writes the record with the per-(warp, telescope) atomics of record_hits.
-// Measured on GB300: 4-8 % less time per launch of the plain FP32 path,
-// 5-7 % with the transmission draw, 1-2 % with spectra, 12-14 % in FP64
-// (where the record's division and products run on the FP64 pipe).
+// (The bound on a step's azimuths that cher_hits.cu uses was tried for the
+// curved atmosphere too: at 70 deg, 10 bunches a step, it costs more than it
+// saves, 79 -> 133 us per 5e4 steps.)
 constexpr int kRing = 64;
 
 template <class R, int BLOCK, bool TR, int FB, bool DS, bool CV>
@@ -114,7 +116,7 @@ __host__ __device__ constexpr size_t segd_offset() {
     return (sizeof(Seg<R>) * BLOCK + sizeof(int) * (BLOCK + 1 + 32) + 15) & ~size_t(15);
 }
 
-// the crossing queue of the hits kernels, after the spectra (DS)
+// the crossing queue of the curved hits kernels, after the spectra (DS)
 template <class R, int BLOCK, bool DS>
 __host__ __device__ constexpr size_t ring_offset() {
     return segd_offset<R, BLOCK>() + (DS ? sizeof(SegD<R>) * BLOCK : 0);
@@ -203,9 +205,6 @@ __device__ __forceinline__ void gen_prop(const KParams &p) {
                            __ldg(p.ekin + i), static_cast<double>(load_dir<R>(p.uz, i)), y, pxyd);
             }
             nb = y.nb;
-            if constexpr (MODE == MODE_HITS) {
-                if (p.prof && nb > 0) profile_step<R>(p, i, static_cast<R>(y.N));
-            }
             ++st_steps;
             st_emit += (nb > 0);
             st_inval += !y.valid;

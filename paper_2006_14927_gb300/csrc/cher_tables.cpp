@@ -598,8 +598,9 @@ void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
 }
 
 void table_slopes(const HostTables &T, double &per_q, double &per_h) {
-    // (rows shared out over threads: a 4000 x 256 table takes a few ms otherwise)
-    const int nthr = std::max(1, std::min(16, T.H / 64));
+    // (a large table's rows are shared out over threads: 4000 x 256 takes 3 ms
+    // otherwise; 1000 x 64 takes less than the threads' start)
+    const int nthr = static_cast<size_t>(T.H) * T.Z < 300000 ? 1 : std::min(16, T.H);
     std::vector<double> mq(nthr, 0.0), mh(nthr, 0.0);
     auto rows = [&](int t) {
         double q = 0.0, h = 0.0;
