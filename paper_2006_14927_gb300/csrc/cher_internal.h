@@ -156,8 +156,8 @@ struct KParams {
     // scheduling
     unsigned *tile_counter;               // NULL: one CTA per tile
     int64_t n_tiles;
-    // the hits kernel's warps take `per_claim` groups of `group` steps at once
-    int32_t group, per_claim;
+    // the hits kernel's warps take groups of `group` steps
+    int32_t group;
     uint32_t n_groups;
     // adjoint screening: frozen bunch counts (NULL: this launch's, written to
     // y_nb), list of (step, bunch) pairs
