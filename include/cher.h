@@ -202,9 +202,9 @@ typedef struct cher_output {
     unsigned long long *stats;   /* [CHER_NSTATS] */
 } cher_output;
 
-/* The whole hot path (a1-a5) for n steps in one launch: a persistent,
- * tile-scheduled kernel whose CTAs pull tiles of steps from an atomic queue
- * in the context's scratch word.  Asynchronous on `stream`; the return value
+/* The whole hot path (a1-a5) for n steps in one launch: a persistent kernel
+ * whose warps (in a curved atmosphere, CTAs) pull groups of steps from an
+ * atomic queue in the context's scratch word.  Asynchronous on `stream`; the return value
  * reports argument checks and the launch only.  Errors: CHER_EINVAL,
  * CHER_ESTATE, CHER_ERANGE (n > 2^40), CHER_ECUDA. */
 cher_status cher_generate_propagate(cher_ctx *ctx, const cher_tracks *tracks,
@@ -366,11 +366,9 @@ cher_status cher_sync_status(cher_ctx *ctx, const cher_output *out,
                              unsigned long long *stats_host, void *stream);
 
 /* Launch shape of cher_generate_propagate.  block_threads in {128, 256,
- * 512} is also the number of steps per tile; ctas_per_sm in 0..10 sets the
- * persistent grid (0 = one CTA per tile, no persistence; above 8 only with
- * 128-step tiles in the FP32 path, which has builds for 9 and 10 CTAs per SM
- * with fewer registers per thread; other launches cap at what fits).  A
- * new context starts at 128 / 8 (32 resident warps per SM); cher_autotune
+ * 512} is also the largest number of steps per tile of the kernels that work
+ * in tiles; ctas_per_sm in 0..10 sets the persistent grid (0 = no persistence),
+ * capped at what fits.  A new context starts at 128 / 8 (32 resident warps per SM); cher_autotune
  * measures the shapes on the caller's input and keeps the fastest.  Errors:
  * CHER_EINVAL. */
 cher_status cher_set_launch(cher_ctx *ctx, int32_t block_threads,

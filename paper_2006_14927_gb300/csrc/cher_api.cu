@@ -396,12 +396,14 @@ struct Shape {
     size_t smem = 0;
 };
 
+// a tile's few steps still fill the four warps of its CTA
+constexpr int kMinTile = 4;
+
 cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int ctas_per_sm,
                  unsigned *counter, Shape &s) {
     s.block = (p.disp_k > 0 || p.earth_radius > 0.0) ? cher::kDispBlock : c->block;
     s.kmode = cher::kernel_mode(mode, p);
     s.smem = cher::kernel_smem_bytes(fp32, s.block, s.kmode, p);
-    p.n_tiles = (p.n + s.block - 1) / s.block;
     p.tile_counter = nullptr;
     if (cher::kernel_prepare(fp32, s.block, s.kmode, s.smem) != cudaSuccess) {
         cudaGetLastError();
@@ -410,6 +412,22 @@ cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int c
     const int fit = cher::kernel_max_ctas_per_sm(fp32, s.block, s.kmode, s.smem);
     const int64_t ctas = int64_t(std::max(1, std::min(ctas_per_sm > 0 ? ctas_per_sm : fit, fit))) *
                          c->num_sms;
+    // Steps per tile: one per thread of a large launch, fewer where whole
+    // blocks would leave SMs idle, down to one wave of CTAs (us per launch with
+    // one per thread -> now: trace of 300 / 3e4 steps FP32 28 -> 9 / 37 -> 20,
+    // 3000 steps FP64 128 -> 37; curved hits, 5e4 steps FP32 31 -> 28, 3000
+    // FP64 84 -> 45; a second or fourth wave of smaller tiles is slower, 22 and
+    // 25 on the 3e4).  A trace, whose CTAs serve one tile each, takes up to
+    // four even waves of at most half a block (1e5 steps FP32 58 -> 51, FP64
+    // 770 -> 710; at 1e6 steps half blocks lose, 449 against 436).
+    p.tile = s.block;
+    if (mode != cher::MODE_YIELD) {
+        const int64_t half = ctas * (s.block / 2);
+        const int64_t waves = counter || p.n > 4 * half ? 1 : (p.n + half - 1) / half;
+        p.tile = static_cast<int32_t>(std::min<int64_t>(
+            s.block, std::max<int64_t>(kMinTile, (p.n + ctas * waves - 1) / (ctas * waves))));
+    }
+    p.n_tiles = (p.n + p.tile - 1) / p.tile;
     int64_t grid = p.n_tiles;
     if (cher::hits_kernel_serves(s.kmode)) {
         // groups of 32 steps, fewer where that would leave warps without

@@ -156,6 +156,7 @@ struct KParams {
     // scheduling
     unsigned *tile_counter;               // NULL: one CTA per tile
     int64_t n_tiles;
+    int32_t tile;                         // steps per tile (at most the block size)
     // the hits kernel's warps take groups of `group` steps
     int32_t group;
     uint32_t n_groups;

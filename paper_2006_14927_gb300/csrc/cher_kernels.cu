@@ -163,12 +163,12 @@ __device__ __forceinline__ void gen_prop(const KParams &p) {
     }
     for (;;) {
         if (tile >= p.n_tiles) break;
-        const int64_t base = tile * BLOCK;
+        const int64_t base = tile * p.tile;
 
         // ---- phase A: one step per thread ----------------------------------
         const int64_t i = base + tid;
         int nb = 0;
-        if (i < p.n) {
+        if (tid < p.tile && i < p.n) {
             // the FP32 path screens the yield in FP32 (same bunch counts as FP64)
             using YT = typename std::conditional<std::is_same<R, float>::value, YieldF,
                                                  Yield>::type;
@@ -247,13 +247,14 @@ __device__ __forceinline__ void gen_prop(const KParams &p) {
         }
         __syncthreads();
         const int excl = v - nb + (warp > 0 ? wsum[warp - 1] : 0);
-        off[tid] = excl;
-        if (tid == BLOCK - 1) off[BLOCK] = excl + nb;
+        // (past the tile's steps no more starts: place `tile` is the total)
+        off[tid] = tid <= p.tile ? excl : 0x7fffffff;
+        if (tid == BLOCK - 1) off[BLOCK] = p.tile == BLOCK ? excl + nb : 0x7fffffff;
         __syncthreads();
-        const int total = off[BLOCK];
+        const int total = off[p.tile];
         if (next < p.n_tiles) {
-            const int64_t ni = next * BLOCK + tid;
-            if (ni < p.n) {
+            const int64_t ni = next * p.tile + tid;
+            if (tid < p.tile && ni < p.n) {
                 prefetch_l2(p.x0 + ni);
                 prefetch_l2(p.y0 + ni);
                 prefetch_l2(p.z0 + ni);
