@@ -573,6 +573,12 @@ cher_status cher_trace_bunches(cher_ctx *ctx, const cher_tracks *tracks,
                                const int64_t *bunch_off, const cher_trace *out,
                                void *stream);
 
+/* Zeros in all n_bunches entries of the arrays and -1 in status (what a
+ * bunch shows that no offset covers), one launch, asynchronous on `stream`.
+ * Errors: CHER_EINVAL, CHER_ECUDA. */
+cher_status cher_clear_trace(cher_ctx *ctx, cher_precision prec, const cher_trace *out,
+                             void *stream);
+
 /* Copy the double-precision tables of the context to host arrays:
  * eta[n_fine], ax[n_heights * n_zenith], al[n_heights * n_zenith]
  * (row-major, height first); any pointer may be NULL.  Errors:

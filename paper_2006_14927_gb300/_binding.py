@@ -132,6 +132,7 @@ SIGNATURES = {
     "cher_segment_yield": (_S, [_P, ctypes.POINTER(Tracks), _S, _P, _P, _P]),
     "cher_trace_bunches": (_S, [_P, ctypes.POINTER(Tracks), ctypes.c_uint64, _S, _P,
                                 ctypes.POINTER(Trace), _P]),
+    "cher_clear_trace": (_S, [_P, _S, ctypes.POINTER(Trace), _P]),
     "cher_get_tables": (_S, [_P, _P, _P, _P]),
     "cher_build_curved_tables_host": (_S, [ctypes.POINTER(Atmosphere), ctypes.c_double,
                                            ctypes.c_double, ctypes.c_int32, ctypes.c_int32,
@@ -437,13 +438,13 @@ class Context:
         nbt = int(bunch_off[-1].item())
         dev = dev_tracks["x0"].device
         dt = torch.float32 if precision == CHER_FP32_BULK else torch.float64
-        pos = torch.zeros((nbt, 4), dtype=dt, device=dev)
-        tim = torch.zeros((nbt, 4), dtype=dt, device=dev)
-        status = torch.full((nbt,), -1, dtype=torch.int32, device=dev)
-        nhit = torch.zeros(nbt, dtype=torch.int32, device=dev)
-        first = torch.zeros(nbt, dtype=torch.int32, device=dev)
+        pos = torch.empty((nbt, 4), dtype=dt, device=dev)
+        tim = torch.empty((nbt, 4), dtype=dt, device=dev)
+        status, nhit, first = (torch.empty(nbt, dtype=torch.int32, device=dev) for _ in range(3))
         tr = Trace(pos.data_ptr(), tim.data_ptr(), status.data_ptr(), nhit.data_ptr(),
                    first.data_ptr(), nbt)
+        _check(lib().cher_clear_trace(self._h, int(precision), ctypes.byref(tr),
+                                      ctypes.c_void_p(_stream_ptr(None))), "cher_clear_trace")
         t = self.tracks_struct(dev_tracks, track_base)
         _check(lib().cher_trace_bunches(self._h, ctypes.byref(t), ctypes.c_uint64(seed),
                                         int(precision), bunch_off.data_ptr(), ctypes.byref(tr),

@@ -1150,6 +1150,20 @@ cher_status cher_trace_bunches(cher_ctx *c, const cher_tracks *t, uint64_t seed,
     return launch(c, p, fp32, cher::MODE_TRACE, false, stream);
 }
 
+cher_status cher_clear_trace(cher_ctx *c, cher_precision prec, const cher_trace *out,
+                             void *stream) {
+    if (!c || !out || out->n_bunches < 0) return CHER_EINVAL;
+    if (prec != CHER_FP64 && prec != CHER_FP32_BULK) return CHER_EINVAL;
+    if (!check_device(c)) return CHER_EINVAL;
+    if (out->n_bunches == 0) return CHER_OK;
+    if (!out->pos || !out->tim || !out->status || !out->nhit || !out->first_hit) return CHER_EINVAL;
+    if (cher::clear_trace(prec == CHER_FP32_BULK, *out, c->num_sms, stream) != cudaSuccess) {
+        cudaGetLastError();
+        return CHER_ECUDA;
+    }
+    return CHER_OK;
+}
+
 cher_status cher_get_tables(const cher_ctx *c, double *eta, double *ax, double *al) {
     if (!c) return CHER_EINVAL;
     if (!c->built) return CHER_ESTATE;

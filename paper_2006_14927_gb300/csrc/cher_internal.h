@@ -278,6 +278,8 @@ inline int kernel_mode(int mode, const KParams &p) {
     if (p.earth_radius > 0.0) m |= kCurvBit;
     return m;
 }
+// Zeros in the trace arrays, status -1.
+cudaError_t clear_trace(bool fp32, const cher_trace &t, int num_sms, void *stream);
 // The fallback pass over the queued bunches (after a MODE_HITS launch with
 // fb_q > 0, on the same stream; reads the queue's count on the device).
 cudaError_t launch_fallback(bool fp32, bool tr, bool disp, const KParams &p, int num_sms,

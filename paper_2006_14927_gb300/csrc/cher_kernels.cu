@@ -515,6 +515,22 @@ __global__ void __launch_bounds__(128) k_fallback(const KParams p) {
     }
 }
 
+// The trace arrays as a bunch that nothing traces leaves them: zeros, status
+// -1.  One pass of stores over 44 bytes (FP32) a bunch instead of a launch for
+// each of the five arrays, which the host could not issue as fast as they ran
+// (yields and trace of 3e4 steps: 223 -> 199 us from call to result).
+template <class R>
+__global__ void k_clear_trace(const cher_trace t) {
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; b < t.n_bunches; b += stride) {
+        store4<R>(t.pos, b, R(0), R(0), R(0), R(0));
+        store4<R>(t.tim, b, R(0), R(0), R(0), R(0));
+        t.status[b] = -1;
+        t.nhit[b] = 0;
+        t.first_hit[b] = 0;
+    }
+}
+
 template <class R, int BLOCK>
 size_t smem_bytes(const KParams &p) {
     size_t b = segd_offset<R, BLOCK>();
@@ -734,6 +750,15 @@ int kernel_max_ctas_per_sm(bool fp32, int block, int mode, size_t smem) {
     if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, block, smem) != cudaSuccess)
         return 0;
     return n;
+}
+
+cudaError_t clear_trace(bool fp32, const cher_trace &t, int num_sms, void *stream) {
+    const int grid = static_cast<int>(
+        std::min<int64_t>((t.n_bunches + 255) / 256, int64_t(num_sms) * 8));
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (fp32) k_clear_trace<float><<<grid, 256, 0, s>>>(t);
+    else k_clear_trace<double><<<grid, 256, 0, s>>>(t);
+    return cudaGetLastError();
 }
 
 cudaError_t kernel_launch(bool fp32, int block, int mode, int grid, size_t smem,
