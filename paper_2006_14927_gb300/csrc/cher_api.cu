@@ -442,8 +442,6 @@ cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int c
     if (counter && grid > ctas) {
         grid = ctas;
         p.tile_counter = counter;
-    } else if (counter && !cher::hits_kernel_serves(s.kmode)) {
-        p.tile_counter = counter;
     }
     if (grid > 0x7fffffff || (p.tile_counter && p.n_tiles > 0xf0000000ll)) return CHER_ERANGE;
     s.grid = static_cast<int>(grid);
