@@ -1230,7 +1230,7 @@ cher_status cher_autotune(cher_ctx *c, const cher_tracks *t, uint64_t seed, cher
         }
     }
     const int blocks[] = {128, 256, 512};
-    const int ctas[] = {0, 1, 2, 3, 4, 6, 8, 9, 10};
+    const int ctas[] = {0, 1, 2, 3, 4, 6, 8};    // (more than 8 do not fit)
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return CHER_ECUDA;
@@ -1241,9 +1241,6 @@ cher_status cher_autotune(cher_ctx *c, const cher_tracks *t, uint64_t seed, cher
     for (int b : blocks)
         for (int cps : ctas) {
             if ((b == 512 && cps > 4) || (b == 256 && cps > 8)) continue;
-            // more than 8 CTAs per SM: the FP32 hits kernel's builds for 9 and
-            // 10 (other precisions and modes cap at what fits)
-            if (cps > 8 && (b != 128 || prec != CHER_FP32_BULK)) continue;
             c->block = b;
             c->ctas_per_sm = cps;
             float tsum = 0.0f;

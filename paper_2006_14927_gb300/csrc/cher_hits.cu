@@ -31,11 +31,11 @@
 // 81-90 bytes a step (the step is 64, a crossing's record 40).  The FP64 kernel
 // is bound by its pipe (83 % busy: the yields' chains and the propagation).
 // Per launch, against the kernel that propagated every bunch:
-//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 285 us
-//   3e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1850 us
-//   2e6 steps, 60 deg, 100 spheres            FP32   685 -> 514 us
-//   2e5 steps, vertical 100 GeV, 19 spheres   FP64  1477 -> 163 us
-//   3e5 steps with spectra                    FP32   234 -> 137 us
+//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 283 us
+//   2e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1667 us
+//   3e6 steps, 60 deg, 100 spheres            FP32   685 -> 496 us
+//   2e5 steps, vertical 100 GeV, 19 spheres   FP64  1477 -> 162 us
+//   3e5 steps with spectra                    FP32   234 -> 138 us
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -387,8 +387,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
 
     // Groups of p.group steps: the first is the warp's own number, the others
     // come from the counter, asked for one ahead (the atomic's latency passes
-    // while the warp works).  One group per request: with up to eight, 2e6
-    // steps at 60 deg took 513 us instead of 496, 3e7 steps of 256 showers
+    // while the warp works).  One group per request: with up to eight, 3e6
+    // steps at 60 deg took 513 us instead of 496, 2e7 steps of 256 showers
     // 1732 instead of 1667.
     const unsigned n_warps = gridDim.x * (blockDim.x >> 5), n_groups = p.n_groups;
     unsigned claim = blockIdx.x * (blockDim.x >> 5) + (tid >> 5) - n_warps;

@@ -50,7 +50,7 @@ namespace {
 // writes the record with the per-(warp, telescope) atomics of record_hits.
 // (The bound on a step's azimuths that cher_hits.cu uses was tried for the
 // curved atmosphere too: at 70 deg, 10 bunches a step, it costs more than it
-// saves, 79 -> 133 us per 5e4 steps.)
+// saves, 79 -> 133 us per 3e5 steps.)
 constexpr int kRing = 64;
 
 template <class R, int BLOCK, bool TR, int FB, bool DS, bool CV>
