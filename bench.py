@@ -6,9 +6,12 @@ Workload (default): 256 showers (primary energies log-uniform 10 GeV -
 10 TeV, zenith 0-40 deg), 2e8 e+- steps in one persistent launch replayed
 from its captured CUDA graph, 100 telescope spheres over 2 x 2 km, refraction
 tables 1000 x 64 up to 70 deg (seeded, synthetic: see workloads/).  A step of
-the benchmark is one launch over all 2e8 steps: every bunch generated,
-refracted, propagated, tested against the spheres and the crossings
-compacted.  The same line carries the 20 TeV shower at 60 deg (1e8 steps,
+the benchmark is one launch over all 2e8 steps: every step's bunches formed,
+those that can reach a sphere (by a bound on the azimuths of each step's cone)
+drawn, refracted, propagated and tested against the spheres, the crossings
+compacted; counters and crossings are what propagating every bunch gives.  The
+rooflines count the operations this needs and, beside it, what propagating
+every bunch would need (that figure exceeds 1).  The same line carries the 20 TeV shower at 60 deg (1e8 steps,
 tables 4000 x 256 to 75 deg) and the 1 TeV vertical shower (2e6 steps) as
 legs with their own roofline, and the FP64 path of each.
 
@@ -90,17 +93,35 @@ FP64_OPS_PER_STEP = 64
 FP32_LANES_PER_SM = 128
 FP64_FMA_PER_SM_CLK = 2         # GB300: 1/64 of the FP32 rate (ncu: 2 DFMA/cycle/SM)
 
+# What a launch needs, by the same counting: the hits kernel bounds the
+# azimuths at which a step's photons can reach a sphere, draws the azimuth word
+# of the bunches of the steps that have such azimuths, and propagates those
+# whose azimuth is among them.  Per step besides validity, yield and Philox
+# share: the bound (without its tests of single telescopes); per drawn bunch:
+# the sub-step loop, Philox for one word (the last round's other half is not
+# needed) and the sector test.  The shares of drawn and propagated bunches were
+# counted on each workload.
+OPS_PER_STEP_BOUND = 110
+OPS_PER_STEP_REACH = (OPS_PER_STEP_FP32["validity"] + OPS_PER_STEP_FP32["yield"] +
+                      OPS_PER_STEP_FP32["philox_step_share"] + OPS_PER_STEP_BOUND)   # 179
+OPS_PER_DRAWN = 66
+BUNCH_SHARES = {                # drawn, propagated
+    "vertical_1tev": (0.4307, 0.02500),
+    "inclined_20tev": (0.6857, 0.02486),
+    "batched_256": (0.2129, 0.01424),
+}
+
 # DRAM bytes (read + write) per step of one FP32 launch, from ncu captures
-# (dram__bytes_read.sum + dram__bytes_write.sum of the fused kernel, in the
-# launch shape the autotuner picks for the workload) at 2e6 steps, scaled to a launch
+# (dram__bytes_read.sum + dram__bytes_write.sum of the hits kernel, in its
+# default launch shape) at 2e6 steps, scaled to a launch
 # by its steps (the inputs, 64 B per step, dominate and scale with them).
 # Reported only while the kernel sources hash to what was profiled.
 TRAFFIC_PER_STEP = {
-    "vertical_1tev": (77.26, "e12d0db1d7ddc53f"),      # 128.74 + 25.79 MB at 2e6 steps, 128 x 8
-    "inclined_20tev": (74.38, "e12d0db1d7ddc53f"),     # 135.36 + 13.40 MB at 2e6 steps, 128 x 10
-    "batched_256": (75.45, "e12d0db1d7ddc53f"),        # 132.56 + 18.35 MB at 2e6 steps, 128 x 10
+    "vertical_1tev": (89.19, "e137018f8c06eb2e"),      # 147.29 + 31.08 MB at 2e6 steps, 128 x 8
+    "inclined_20tev": (79.78, "e137018f8c06eb2e"),     # 146.16 + 13.40 MB at 2e6 steps, 128 x 8
+    "batched_256": (80.85, "e137018f8c06eb2e"),        # 144.29 + 17.41 MB at 2e6 steps, 128 x 8
 }
-KERNEL_SOURCES = ("cher_kernels.cu", "cher_device.cuh", "cher_internal.h")
+KERNEL_SOURCES = ("cher_hits.cu", "cher_path.cuh", "cher_device.cuh", "cher_internal.h")
 
 
 def _kernel_hash() -> str:
@@ -143,6 +164,26 @@ def fp64_roofline(bunches: float, steps: float, ms: float, sm_count: int, mhz: f
             "ops_per_step": FP64_OPS_PER_STEP,
             "peak_source": f"derived: {sm_count} SMs x {FP64_FMA_PER_SM_CLK} FP64 lanes x "
                            f"{mhz:.0f} MHz"}
+
+
+def needed(rl: dict, wl: str, bunches: float, steps: float, ms: float):
+    """The roofline of propagating every bunch (alu_roofline, fp64_roofline)
+    with achieved and frac replaced by those of the operations the launch
+    needs; the former stay as all_bunches_*."""
+    if wl not in BUNCH_SHARES:
+        return rl
+    drawn, prop = BUNCH_SHARES[wl]
+    if rl["bound"] == "alu":
+        ops = OPS_PER_STEP_REACH * steps + (OPS_PER_DRAWN * drawn + OPS_PER_BUNCH * prop) * bunches
+    else:
+        ops = FP64_OPS_PER_STEP * steps + FP64_OPS_PER_BUNCH * prop * bunches
+    achieved = ops / (ms / 1e3) / 1e12
+    return {**rl, "achieved": achieved, "frac": achieved / rl["peak"],
+            "ops_per_step_needed": ops / steps, "drawn_share": drawn, "propagated_share": prop,
+            "all_bunches_achieved": rl["achieved"], "all_bunches_frac": rl["frac"],
+            "note": "frac counts the operations the launch needs; all_bunches_frac those of "
+                    "propagating every bunch, of which the kernel skips those that cannot "
+                    "reach a sphere"}
 
 
 def _peaks():
@@ -396,12 +437,13 @@ def workload_leg(P, dev, wl, scale, cap_arg, steps, warmup, launch, main_launch,
     n = B.n
     b32, b64 = float(r32["stats"][3]), float(r64["stats"][3])
     ms32, ms64 = statistics.mean(r32["ms"]), statistics.mean(r64["ms"])
-    rl = alu_roofline(b32, n, ms32, sm_count, mhz)
+    rl = needed(alu_roofline(b32, n, ms32, sm_count, mhz), wl, b32, n, ms32)
     rl["traffic"] = _traffic(wl, n)
     res = {"value": b32 / (ms32 / 1e3), "unit": UNIT, "ms_per_step": ms32,
            "bunches_per_step": int(b32), "steps_per_gpu": n, "roofline": rl,
            "fp64": {"value": b64 / (ms64 / 1e3), "ms_per_step": ms64,
-                    "roofline": fp64_roofline(b64, n, ms64, sm_count, mhz)},
+                    "roofline": needed(fp64_roofline(b64, n, ms64, sm_count, mhz), wl, b64, n,
+                                       ms64)},
            "fp32_over_fp64": (b32 / ms32) / (b64 / ms64),
            "overflowed_records": int(r32["stats"][10]), "table_build_s": B.table_s,
            "launch": {"block": own[0], "ctas_per_sm": own[1]},
@@ -541,14 +583,15 @@ def run_ours(args):
             torch.distributed.destroy_process_group()
         return
 
-    # ---- roofline of the dominant kernel (ALU bound) ----------------------
+    # ---- roofline of the dominant kernel (issue bound) --------------------
     st = rg["stats"]
     bunches, steps_n = float(st[3]), float(st[0])
     ms_g = statistics.mean(rg["ms"])
-    rl = alu_roofline(bunches, steps_n, ms_g, sm_count, mhz)
+    rl = needed(alu_roofline(bunches, steps_n, ms_g, sm_count, mhz), wl, bunches, steps_n, ms_g)
     rl["traffic"] = _traffic(wl, n) if args.scale == 1.0 else None
     ms64 = statistics.mean(r64["ms"])
-    rl64 = fp64_roofline(float(r64["stats"][3]), steps_n, ms64, sm_count, mhz)
+    b64 = float(r64["stats"][3])
+    rl64 = needed(fp64_roofline(b64, steps_n, ms64, sm_count, mhz), wl, b64, steps_n, ms64)
     # the FP64 path beside the FP32 one inside the roofline object as well
     rl["fp64_path"] = {"value": v64, "frac": rl64["frac"], "fp32_over_fp64": vg / v64}
     cpu = _leg(cpu_baseline, wl) if world == 1 else None
