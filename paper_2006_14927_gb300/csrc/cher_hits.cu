@@ -422,6 +422,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 i = have ? W.exact[first + lane] : 0;
                 n_exact = first;
             } else {
+                // (the streams' first groups, then their second ones, ...)
+                if (p.streams > 1) cur = cur % p.streams * (n_groups / p.streams) + cur / p.streams;
                 i = int64_t(cur) * p.group + lane;
                 have = lane < p.group && i < p.n;
             }

@@ -157,9 +157,11 @@ struct KParams {
     unsigned *tile_counter;               // NULL: one CTA per tile
     int64_t n_tiles;
     int32_t tile;                         // steps per tile (at most the block size)
-    // the hits kernel's warps take groups of `group` steps
+    // the hits kernel's warps take groups of `group` steps, in order or (a
+    // production profile of several showers) in turn from `streams` equal parts
+    // of the list
     int32_t group;
-    uint32_t n_groups;
+    uint32_t n_groups, streams;
     // adjoint screening: frozen bunch counts (NULL: this launch's, written to
     // y_nb), list of (step, bunch) pairs
     // that land within the read-out radius of a telescope centre

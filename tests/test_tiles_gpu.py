@@ -7,6 +7,7 @@ waves than one.  The same arithmetic per bunch, so bit-equal."""
 import numpy as np
 import pytest
 
+import paper_2006_14927_gb300 as P
 import workloads
 from parity import FP32, FP64, context, gpu_hits, gpu_trace, host_tracks
 
@@ -50,3 +51,45 @@ def test_curved_crossings_of_small_tiles(prec, n):
         for k in r:
             assert np.array_equal(r[k], got[0][1][k]), k
     assert n < 1000 or len(got[0][1]["key"]) > 100
+
+
+@pytest.mark.parametrize("prec,n", [(FP32, 24_321), (FP32, 70_001), (FP64, 25_003)])
+def test_profile_of_showers_taken_in_turn(prec, n):
+    """A production profile of several showers, whose groups the warps take in
+    turn from parts of the list, against each shower in a launch of its own
+    (in order, equal bins combined): the same crossings and counters, and sums
+    that differ by the order of at most n FP64 additions of positive terms."""
+    import torch
+    sc = workloads.vertical_1tev(n=n)
+    ctx, tr = context(sc), host_tracks(sc, prec)
+    rows, edges = 3, [0, n // 5, n // 5 + 7, n]
+    t_ref = np.repeat(sc["t_ref"][:1], rows)
+
+    def run(lo, hi, shower, prof):
+        t = dict(_part(tr, lo, hi), shower=shower[lo:hi])
+        dev = P.device_tracks(t, prec, t_ref=t_ref)
+        out = ctx.alloc_hits(n, prec)
+        ctx.generate_propagate(dev, 7, prec, out, track_base=lo, profile=prof, bin_gcm2=10.0)
+        code, stats = ctx.sync_status(out)
+        assert code == 0
+        return np.asarray(stats), out.records()
+
+    shower = np.repeat(np.arange(rows), np.diff(edges)).astype(tr["shower"].dtype)
+    prof = torch.zeros((rows, 120), dtype=torch.float64, device="cuda")
+    stats, rec = run(0, n, shower, prof)
+    alone, total, recs = torch.zeros_like(prof), 0, []
+    for k in range(rows):
+        one = torch.zeros((rows, 120), dtype=torch.float64, device="cuda")
+        ctx.set_launch(128, 1 if k == 0 else 8)          # fewer warps: full groups, no parts
+        st, r = run(edges[k], edges[k + 1], shower, one)
+        alone += one
+        total = total + st
+        recs.append(r)
+    assert np.array_equal(stats, total)
+    both = {k: np.concatenate([r[k] for r in recs]) for k in rec}
+    at = np.lexsort((both["key"], both["tel"]))
+    for k in rec:
+        assert np.array_equal(rec[k], both[k][at]), k
+    assert prof.sum() > 0
+    bound = n * 2.0 ** -52 * alone
+    assert bool(((prof - alone).abs() <= bound).all())
