@@ -117,9 +117,9 @@ BUNCH_SHARES = {                # drawn, propagated
 # by its steps (the inputs, 64 B per step, dominate and scale with them).
 # Reported only while the kernel sources hash to what was profiled.
 TRAFFIC_PER_STEP = {
-    "vertical_1tev": (89.19, "e137018f8c06eb2e"),      # 147.29 + 31.08 MB at 2e6 steps, 128 x 8
-    "inclined_20tev": (79.78, "e137018f8c06eb2e"),     # 146.16 + 13.40 MB at 2e6 steps, 128 x 8
-    "batched_256": (80.85, "e137018f8c06eb2e"),        # 144.29 + 17.41 MB at 2e6 steps, 128 x 8
+    "vertical_1tev": (89.06, "fd01f26aca17b9e1"),      # 147.32 + 30.81 MB at 2e6 steps, 128 x 8
+    "inclined_20tev": (80.01, "fd01f26aca17b9e1"),     # 146.24 + 13.77 MB at 2e6 steps, 128 x 8
+    "batched_256": (80.87, "fd01f26aca17b9e1"),        # 144.29 + 17.45 MB at 2e6 steps, 128 x 8
 }
 KERNEL_SOURCES = ("cher_hits.cu", "cher_path.cuh", "cher_device.cuh", "cher_internal.h")
 
