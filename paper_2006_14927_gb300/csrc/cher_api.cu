@@ -410,8 +410,10 @@ cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int c
         return CHER_ERANGE;
     }
     const int fit = cher::kernel_max_ctas_per_sm(fp32, s.block, s.kmode, s.smem);
-    const int64_t ctas = int64_t(std::max(1, std::min(ctas_per_sm > 0 ? ctas_per_sm : fit, fit))) *
-                         c->num_sms;
+    // (a mode with its own block size keeps the threads per SM of the set shape:
+    // spectra under 512 x 2 ran as 128 x 2, 64 ms instead of 37 for 2e8 steps)
+    const int want = ctas_per_sm > 0 ? ctas_per_sm * std::max(1, c->block / s.block) : fit;
+    const int64_t ctas = int64_t(std::max(1, std::min(want, fit))) * c->num_sms;
     // Steps per tile: one per thread of a large launch, fewer where whole
     // blocks would leave SMs idle, down to one wave of CTAs (us per launch with
     // one per thread -> now: trace of 300 / 3e4 steps FP32 28 -> 9 / 37 -> 20,
