@@ -388,26 +388,26 @@ __global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
             Y = o.Y.v;
             t = o.t.v;
             w = o.w.v;
-            Xf = static_cast<float>(o.X.v);
-            Yf = static_cast<float>(o.Y.v);
+            Xf = static_cast<float>(X - A.k.cull.ox);
+            Yf = static_cast<float>(Y - A.k.cull.oy);
         }
         double gX = 0, gY = 0, gt = 0, gw = 0;
         bool any = false;
-        // Most telescopes are out of reach, which is seen in FP32 (with room
-        // for its rounding).  Every lane looks for its own next one first, so
+        // Most telescopes are out of reach, which is seen in FP32 from the
+        // middle of the array (with room for its rounding).  Every lane looks for its own next one first, so
         // that the lanes' FP64 work on theirs runs together.
         for (int k = live ? 0 : n_tel;; ++k) {
             for (; k < n_tel; ++k) {
                 const float4 C = __ldg(A.k.cull.tel + k);
-                if (fabsf(Xf - C.x) < A.reach && fabsf(Yf - C.y) < A.reach) break;
+                if (!(fabsf(Xf - C.x) >= A.reach) && !(fabsf(Yf - C.y) >= A.reach)) break;
             }
             if (!__any_sync(kFull, k < n_tel)) break;
             if (k >= n_tel) continue;
             double tx, ty;
             if constexpr (std::is_same<T, float>::value) {
-                const float4 C = __ldg(A.k.cull.tel + k);
-                tx = C.x;
-                ty = C.y;
+                const float4 Tt = __ldg(static_cast<const float4 *>(A.k.tel) + k);
+                tx = Tt.x;
+                ty = Tt.y;
             } else {
                 const double2 Tt = __ldg(static_cast<const double2 *>(A.k.tel) + 2 * k);
                 tx = Tt.x;

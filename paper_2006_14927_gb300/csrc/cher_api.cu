@@ -324,6 +324,17 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
     p.cull.ax_sq = static_cast<float>(1.01 * c->ax_sq);
     p.cull.ax_sh = static_cast<float>(1.01 * c->ax_sh);
     p.cull.words = c->CB.words;
+    p.cull.ox = c->CB.ox;
+    p.cull.oy = c->CB.oy;
+    p.cull.ex = static_cast<float>(c->CB.ex);
+    p.cull.ey = static_cast<float>(c->CB.ey);
+    // Rounding of coordinates, four of at most half an ulp each (2.4e-7 of
+    // their size): the bound's own, relative to the middle of the array, and
+    // in the FP32 path the ground points', which are absolute; the FP64 path's
+    // ground points round 2^-29 times as much.
+    const double far = std::fabs(c->CB.ox) + std::fabs(c->CB.oy);
+    p.cull.err_m = fp32 ? 5e-7f : 2.5e-7f;
+    p.cull.err_0 = static_cast<float>((fp32 ? 2.5e-7 : 8e-16) * far);
     p.cull.x0 = static_cast<float>(c->CB.x0);
     p.cull.y0 = static_cast<float>(c->CB.y0);
     p.cull.inv_bx = static_cast<float>(c->CB.inv_bx);
@@ -652,14 +663,15 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
             tel32[4 * k + m] = static_cast<float>(v[m]);
         }
     }
-    // the telescopes for the hits kernel's bound (radii rounded up)
+    // the telescopes for the hits kernel's bound, from the middle of the array
+    // (radii rounded up)
     cher::build_center_bins(c->tel.data(), static_cast<int32_t>(nt), c->CB);
     std::vector<float> ctel(nt * 4);
     c->cull_rmax = c->cull_zmax = 0.0;
     for (size_t m = 0; m < nt; ++m) {
         const cher_telescope &q = c->tel[m];
-        ctel[4 * m] = static_cast<float>(q.x);
-        ctel[4 * m + 1] = static_cast<float>(q.y);
+        ctel[4 * m] = static_cast<float>(q.x - c->CB.ox);
+        ctel[4 * m + 1] = static_cast<float>(q.y - c->CB.oy);
         ctel[4 * m + 2] = static_cast<float>(q.z);
         ctel[4 * m + 3] = static_cast<float>(q.r * (1.0 + 1e-6));
         c->cull_rmax = std::max(c->cull_rmax, q.r * (1.0 + 1e-6));
@@ -1353,6 +1365,7 @@ cher_status readout(cher_ctx *c, const cher_tracks *t, uint64_t seed, cher_preci
     double far = 0.0;
     for (const cher_telescope &q : c->tel) far = std::max({far, std::fabs(q.x), std::fabs(q.y)});
     A.reach = static_cast<float>(6.0 * sigma * 1.0001 + 1e-3 + 1e-6 * far);
+    if (!std::isfinite(A.reach)) A.reach = std::nanf("");
     A.S = c->d_SU;
     A.U = c->d_SU + n_tel;
     A.sens = c->d_sens;

@@ -76,7 +76,8 @@ static_assert(kQueue >= 31 + 32 * kPer, "a window's bunches fit behind the queue
 // times the angle between the step and the line), of g A_x and of delta over
 // the cone (their derivatives along the cone, at the largest zenith on it,
 // times the cone's angle), of n along the step, and the arithmetic (5 cm plus
-// 1e-5 rad sec^2).  p = cos_c u + sin_c (cos phi e1 + sin phi e2), and with
+// 1e-5 rad sec^2, and the rounding of the coordinates, which grows with them:
+// KParams::Cull).  p = cos_c u + sin_c (cos phi e1 + sin phi e2), and with
 // a = V.u, b = (V.e1, V.e2)
 //     |V x p| >= | sin_c a (cos phi, sin phi) - cos_c b |
 // (the distance of the two directions' gnomonic projections), so a crossing
@@ -115,9 +116,13 @@ struct Box {
 // may be dropped on its way to the ground.  (Written without early returns:
 // the lanes of a group stay together.)
 template <int MODE, bool DS>
-__device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, float dz0, float L,
-                                          float ux, float uy, float uz, float eta, float sinc_lo,
-                                          float sinc_hi, Ring &G, Near &N, Box &B) {
+__device__ __forceinline__ int ring_setup(const KParams &p, double x0d, double y0d, float dz0,
+                                          float L, float ux, float uy, float uz, float eta,
+                                          float sinc_lo, float sinc_hi, Ring &G, Near &N, Box &B) {
+    // from the middle of the array, and the rounding of coordinates
+    const float x0 = __double2float_rn(x0d - p.cull.ox), y0 = __double2float_rn(y0d - p.cull.oy);
+    const float err = p.cull.err_m * (fmaxf(fabsf(x0), p.cull.ex) + fmaxf(fabsf(y0), p.cull.ey)) +
+                      p.cull.err_0;
     const float su2 = ux * ux + uy * uy;
     // the step points down, is a unit vector, and its cone is narrow
     bool ok = (uz < 0.0f) & (fabsf(su2 + uz * uz - 1.0f) <= 4e-6f) & (sinc_hi <= 0.25f);
@@ -178,7 +183,7 @@ __device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, 
     if (DS) dA += fabsf(A) * (0.1f + (k_hi - k_lo));
     const float mA = 1.02f * (fabsf(A) + dA) * sec2 * (3.0f * sec2 - 2.0f) * th + g * su * dA;
     const float bs = bend * sec_hi;
-    const float mo = 0.06f + half * (sinc_hi + 1.1f * bs) + mA;
+    const float mo = 0.06f + err + half * (sinc_hi + 1.1f * bs) + mA;
     const float mw = (1e-5f + 2.2f * bend * th) * sec2 + (1.1f * drat + dkap) * sec_hi + bs * bs;
     const float fac = 1.002f + 1.5f * bs;
     G.a = make_float4(X0, Y0, dzm, sm);
@@ -192,7 +197,7 @@ __device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, 
     // (across) of the axis's point per metre of height, so in a box around it
     const float r_max = MODE == MODE_SCREEN ? p.cull.r_cut : p.cull.r_max;
     const float dist = dzm + half;
-    const float slack = dist * sec2 * mw + mA + 1.0f + 0.02f * L +
+    const float slack = dist * sec2 * mw + mA + err + 1.0f + 0.02f * L +
                         (1.01f * r_max + p.cull.z_max) * sec_hi;
     const float across = 1.03f * th * dist * sec_hi, along = across * sec_hi;
     const float ca = fabsf(e1y), sa = fabsf(e1x);        // the step's azimuth
@@ -489,8 +494,7 @@ __device__ __forceinline__ void hits(const KParams &p) {
                     } else {
                         s_lo = s_hi = sqrtf(d2f_rn(y.s2));
                     }
-                    kind = ring_setup<MODE, DS>(p, __double2float_rn(__ldg(p.x0 + i)),
-                                                __double2float_rn(__ldg(p.y0 + i)),
+                    kind = ring_setup<MODE, DS>(p, __ldg(p.x0 + i), __ldg(p.y0 + i),
                                                 __double2float_rn(z0) - p.f.h_obs,
                                                 __double2float_rn(len), ux, uy, uzf,
                                                 eta, s_lo, s_hi,

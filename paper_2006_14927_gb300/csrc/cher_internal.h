@@ -64,8 +64,12 @@ cher_status build_grid(const cher_telescope *tel, int32_t n_tel, double theta_ma
                        HostGrid &g);
 // Prefix masks of the telescopes' centres over kCullBins bins per axis
 // (KParams::cull), and the largest slopes of ax over the table's cells.
+// Coordinates are taken from the middle (ox, oy) of the centres' box, whose
+// half sizes are ex, ey: single precision resolves the array wherever the
+// caller's coordinates have their origin.
 struct HostBins {
     int32_t words = 0;
+    double ox = 0, oy = 0, ex = 0, ey = 0;
     double x0 = 0, y0 = 0, inv_bx = 0, inv_by = 0;
     std::vector<uint32_t> masks;          // [2][kCullBins + 1][words]
 };
@@ -132,9 +136,14 @@ struct KParams {
     // correction (per sin^2 of the zenith, per metre of height), the
     // telescopes (float4 x, y, z, r) with the largest radius and height, and
     // for boxes of their centres the prefix masks of kCullBins bins per axis:
-    // word w of entry b holds the telescopes 32 w .. 32 w + 31 in bins < b
+    // word w of entry b holds the telescopes 32 w .. 32 w + 31 in bins < b.
+    // Telescopes and bins are relative to (ox, oy), the middle of the array,
+    // which is subtracted from a step's place in FP64; err_m (|x| + |y|) +
+    // err_0 bounds the rounding of both kernels' coordinates (base_params)
     struct Cull {
         const float2 *tab32;
+        double ox, oy;
+        float ex, ey, err_m, err_0;
         float ax_sq, ax_sh;
         int words;
         float x0, y0, inv_bx, inv_by, r_max, z_max, r_cut;
@@ -242,6 +251,7 @@ struct AdjParams {
     const int32_t *nb;
     double sigma, inv_2s2, norm, rcut2;
     float reach;                   // 6 sigma and the rounding of an FP32 difference
+                                   // (NaN: no telescope is out of reach)
     double *S, *U;                 // [n_tel] read-out sums
     const double *gD, *gT;         // [n_tel] upstream gradients
     double *grad_atm;              // [15]: a_0..a_4, b_0..b_4, c_0..c_4

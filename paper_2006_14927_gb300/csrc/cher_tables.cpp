@@ -581,16 +581,18 @@ void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
             lo = std::min(lo, v);
             hi = std::max(hi, v);
         }
+        const double mid = 0.5 * lo + 0.5 * hi, half = 0.5 * hi - 0.5 * lo;
+        (axis ? b.oy : b.ox) = mid;
+        (axis ? b.ey : b.ex) = half;
         // room on both sides for single-precision bin indices
-        const double mag = 1.0 + 1e-5 * std::max(std::fabs(lo), std::fabs(hi));
-        lo -= mag;
-        const double inv = kCullBins / (hi + mag - lo);
-        (axis ? b.y0 : b.x0) = lo;
-        (axis ? b.inv_by : b.inv_bx) = inv;
+        const double edge = half + (1.0 + 1e-5 * half);
+        (axis ? b.y0 : b.x0) = -edge;
+        (axis ? b.inv_by : b.inv_bx) = 0.5 * kCullBins / edge;
         uint32_t *m = b.masks.data() + axis * size_t(kCullBins + 1) * b.words;
         for (int k = 0; k < n_tel; ++k) {
+            const double at = ((axis ? tel[k].y : tel[k].x) - mid) / edge;      // in (-1, 1)
             const int bin = std::min(kCullBins - 1,
-                                     static_cast<int>(((axis ? tel[k].y : tel[k].x) - lo) * inv));
+                                     static_cast<int>(0.5 * kCullBins * (at + 1.0)));
             for (int e = bin + 1; e <= kCullBins; ++e)
                 m[size_t(e) * b.words + k / 32] |= 1u << (k % 32);
         }
