@@ -190,7 +190,10 @@ __device__ __forceinline__ int ring_setup(const KParams &p, double x0d, double y
     G.d = make_float4(dx, dy, dz, mo);
     G.u = make_float4(ux, uy, uz, mw);
     G.e = make_float4(e1x, e1y, fac, spread);
-    const float s_lo = fmaxf(su * cch - cu * sinc_hi, 0.0f) * (1.0f - bend);
+    // (rounded down by 1e-6 of itself and 1e-6, as s_hi up: at 83 deg 1 / cos
+    // moves by 66 times the sine's relative error)
+    const float su_lo = tilted ? su2 * isu * 0.999999f : 0.0f;
+    const float s_lo = fmaxf(su_lo * cch - cu * sinc_hi - 1e-6f, 0.0f) * (1.0f - bend);
     B.sec_lo = ok ? rsqrtf(1.0f - s_lo * s_lo) * 0.99999f : 0.0f;
     B.sec_hi = ok ? sec_hi : 1e30f;        // (0 .. 1e30: decides no transmission draw)
     // the ring on the ground: within sec^2 th (along the azimuth) and sec th
