@@ -680,7 +680,10 @@ __device__ __forceinline__ void hits(const KParams &p) {
                                 p_lo = exp(-(tau * static_cast<R>(sec.y)));
                                 p_hi = exp(-(tau * static_cast<R>(sec.x)));
                             }
-                            const bool gone = !(u3 < p_hi * R(1.00002));
+                            // (a depth past the precision's range makes the
+                            // probabilities NaN where the zenith is unbounded:
+                            // propagated)
+                            const bool gone = u3 >= p_hi * R(1.00002);
                             const bool stays = u3 < p_lo * R(0.99998);
                             if (gone) atomicAdd(&W.drop[ST_ABSORBED], 1u);
                             pass = !gone && (pass || !stays);

@@ -59,3 +59,27 @@ def test_draw_at_the_cone_s_smallest_zenith(zenith, prec):
         assert want[0] > 0 and want[5] > 0 and want[0] + want[5] == sum(want)
     assert bunches > 8e7
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_draw_with_opaque_nodes(prec):
+    """Optical depths beyond FP32's range (opaque air): upward bunches and
+    those past the tables' edges are counted as such, the rest absorbed."""
+    rng = np.random.Generator(np.random.PCG64(5))
+    n = 4000
+    seg, t_ref = workloads.shower_segments(rng, n, 1.0e6, 0.3, 0.7, 0.0, 0.0, H_OBS)
+    d = rng.normal(size=(n, 3))
+    d /= np.linalg.norm(d, axis=1)[:, None]
+    seg["ux"], seg["uy"], seg["uz"] = d.T.copy()
+    ctx = P.Context(workloads.us_standard_atmosphere(), H_OBS, [[0.0, 0.0, 0.0, 5.0]])
+    ctx.build_refraction_tables(400, 64, 70.0, 60000.0)
+    ctx.set_transmission(_constant_tau(1e39))
+    dev = P.device_tracks(seg, prec, t_ref=t_ref)
+    tr, _ = all_bunches(ctx, dev, n, 3, prec)
+    status = tr["status"].cpu().numpy()
+    out = ctx.alloc_hits(1000, prec)
+    ctx.generate_propagate(dev, 3, prec, out)
+    _, st = ctx.sync_status(out)
+    want = [int((status == s).sum()) for s in range(6)]
+    assert [int(st[i]) for i in (8, 4, 5, 6, 7, 11)] == want
+    assert want[1] > 1000 and want[4] > 1000 and want[5] > 1000 and want[0] == 0
