@@ -50,8 +50,9 @@ class _Readout(torch.autograd.Function):
                              fctx.sigma, fctx.nb)
         da, dp, dd = fctx.dtypes
         va, vp, vd = fctx.devices
-        # (one conversion for the three positions, one for the directions)
-        grads = [*gt[:3].to(device=vp, dtype=dp), *gt[3:].to(device=vd, dtype=dd)]
+        # (converted one by one: a gradient in another type has memory of its own)
+        grads = [g.to(device=vp if m < 3 else vd, dtype=dp if m < 3 else dd)
+                 for m, g in enumerate(gt.unbind(0))]
         return (ga.to(device=va, dtype=da), *grads, None, None, None, None, None, None, None,
                 None)
 
