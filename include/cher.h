@@ -558,7 +558,8 @@ cher_status cher_segment_yield(cher_ctx *ctx, const cher_tracks *tracks,
  *                 4 beyond the zenith range, 5 reached h_obs but lost to
  *                 the atmospheric transmission (no ground point then)
  *   nhit[b], first_hit[b] = number of spheres crossed, lowest index or -1.
- * pos/tim are float (CHER_FP32_BULK) or double (CHER_FP64). */
+ * pos/tim are float (CHER_FP32_BULK) or double (CHER_FP64), 16-byte aligned
+ * (CHER_EINVAL otherwise). */
 typedef struct cher_trace {
     void *pos;
     void *tim;

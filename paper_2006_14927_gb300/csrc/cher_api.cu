@@ -269,6 +269,11 @@ bool tracks_ok(const cher_tracks *t) {
     return true;
 }
 
+// the kernels write a trace's pos and tim 16 bytes at a time
+bool stores_aligned(const cher_trace &t) {
+    return reinterpret_cast<uintptr_t>(t.pos) % 16 == 0 && reinterpret_cast<uintptr_t>(t.tim) % 16 == 0;
+}
+
 cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed, bool fp32) {
     cher::KParams p;
     std::memset(&p, 0, sizeof(p));
@@ -1157,7 +1162,7 @@ cher_status cher_trace_bunches(cher_ctx *c, const cher_tracks *t, uint64_t seed,
     if (!c->built) return CHER_ESTATE;
     if (!check_device(c)) return CHER_EINVAL;
     if (t->n > 0 && (!bunch_off || !out->pos || !out->tim || !out->status || !out->nhit ||
-                     !out->first_hit))
+                     !out->first_hit || !stores_aligned(*out)))
         return CHER_EINVAL;
     const bool fp32 = prec == CHER_FP32_BULK;
     cher::KParams p = base_params(c, t, seed, fp32);
@@ -1177,7 +1182,9 @@ cher_status cher_clear_trace(cher_ctx *c, cher_precision prec, const cher_trace 
     if (prec != CHER_FP64 && prec != CHER_FP32_BULK) return CHER_EINVAL;
     if (!check_device(c)) return CHER_EINVAL;
     if (out->n_bunches == 0) return CHER_OK;
-    if (!out->pos || !out->tim || !out->status || !out->nhit || !out->first_hit) return CHER_EINVAL;
+    if (!out->pos || !out->tim || !out->status || !out->nhit || !out->first_hit ||
+        !stores_aligned(*out))
+        return CHER_EINVAL;
     if (cher::clear_trace(prec == CHER_FP32_BULK, *out, c->num_sms, stream) != cudaSuccess) {
         cudaGetLastError();
         return CHER_ECUDA;
