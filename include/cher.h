@@ -608,7 +608,7 @@ cher_status cher_build_tables_host(const cher_atmosphere *atm, double h_obs,
 /* Measure a few launch shapes of cher_generate_propagate on the given
  * input (which must already be resident) and keep the fastest; if
  * cache_path is not NULL the choice is read from / appended to that file
- * (one line per device name, precision and tile count).  Writes into `out`
+ * (one line per device name, revision of the kernels, precision and tile count).  Writes into `out`
  * while measuring.  Errors as cher_generate_propagate, plus CHER_EINVAL if
  * the cache file is unreadable garbage. */
 cher_status cher_autotune(cher_ctx *ctx, const cher_tracks *tracks,

@@ -1240,8 +1240,11 @@ cher_status cher_autotune(cher_ctx *c, const cher_tracks *t, uint64_t seed, cher
     if (cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) return CHER_ECUDA;
     char tag[512];
     const long long tiles_bucket = static_cast<long long>(std::log2(double(t->n) + 1.0));
-    std::snprintf(tag, sizeof(tag), "%s|%d|%lld|%d|%d", prop.name, static_cast<int>(prec),
-                  tiles_bucket, static_cast<int>(c->tel.size()), c->T.Z);
+    // (the revision of the kernels that are timed: a shape that was found for
+    // others is measured again)
+    constexpr int kTunedKernels = 2;
+    std::snprintf(tag, sizeof(tag), "%s|k%d|%d|%lld|%d|%d", prop.name, kTunedKernels,
+                  static_cast<int>(prec), tiles_bucket, static_cast<int>(c->tel.size()), c->T.Z);
     for (char *q = tag; *q; ++q)
         if (*q == ' ') *q = '_';
     if (cache_path) {
