@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kPairBlock) k_adj_pairs(const AdjParams A) {
         // that the lanes' FP64 work on theirs runs together.
         for (int k = live ? 0 : n_tel;; ++k) {
             for (; k < n_tel; ++k) {
-                const float4 C = __ldg(A.k.cull.tel + k);
+                const float4 C = __ldg(A.k.cull.tel0 + k);
                 if (!(fabsf(Xf - C.x) >= A.reach) && !(fabsf(Yf - C.y) >= A.reach)) break;
             }
             if (!__any_sync(kFull, k < n_tel)) break;

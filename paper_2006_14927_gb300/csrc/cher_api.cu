@@ -42,6 +42,7 @@ struct cher_ctx {
     // the hits kernel's bins of telescope centres and table slopes
     cher::HostBins CB;
     float *d_cull = nullptr;              // the telescopes, then the bins' masks
+    bool crowded = false;                 // launches ask which hits kernel pays (plan)
     double cull_rmax = 0, cull_zmax = 0, ax_sq = 0, ax_sh = 0;
     // scratch: the persistent kernel's tile counter
     unsigned *d_scratch = nullptr;
@@ -347,7 +348,8 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
     p.cull.r_max = static_cast<float>(c->cull_rmax);
     p.cull.z_max = static_cast<float>(c->cull_zmax);
     p.cull.tel = reinterpret_cast<const float4 *>(c->d_cull);
-    p.cull.bins = reinterpret_cast<const uint32_t *>(c->d_cull + 4 * c->tel.size());
+    p.cull.tel0 = p.cull.tel + c->tel.size();
+    p.cull.bins = reinterpret_cast<const uint32_t *>(p.cull.tel0 + c->tel.size());
     // the layered thickness, for the production profile
     for (int l = 0; l < 6; ++l) p.atm.hb[l] = c->atm.h_bound[l];
     for (int l = 0; l < 5; ++l) {
@@ -410,7 +412,11 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
 struct Shape {
     int block = 0, kmode = 0, grid = 0;
     size_t smem = 0;
+    int probe = 0, direct = 0;            // with p.choice: the kernels around the first
+    size_t direct_smem = 0;
 };
+
+constexpr int64_t kProbeSteps = 50000;
 
 // a tile's few steps still fill the four warps of its CTA
 constexpr int kMinTile = 4;
@@ -418,9 +424,10 @@ constexpr int kMinTile = 4;
 cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int ctas_per_sm,
                  unsigned *counter, Shape &s) {
     s.block = (p.disp_k > 0 || p.earth_radius > 0.0) ? cher::kDispBlock : c->block;
-    s.kmode = cher::kernel_mode(mode, p);
+    s.kmode = cher::kernel_mode(mode, p, fp32);
     s.smem = cher::kernel_smem_bytes(fp32, s.block, s.kmode, p);
     p.tile_counter = nullptr;
+    p.choice = nullptr;
     if (cher::kernel_prepare(fp32, s.block, s.kmode, s.smem) != cudaSuccess) {
         cudaGetLastError();
         return CHER_ERANGE;
@@ -465,6 +472,20 @@ cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int c
             p.n_groups = static_cast<uint32_t>((groups + 63) / 64 * 64);   // (equal parts)
         }
         grid = (int64_t(p.n_groups) + wpc - 1) / wpc;
+        // Where the bound of the azimuths may cost more than it saves, 1216
+        // steps spread over the list are asked first, and of the two kernels
+        // that follow one ends at once (the FP64 path always gains)
+        if (counter && fp32 && mode == cher::MODE_HITS && p.n >= kProbeSteps &&
+            (c->crowded || p.fb_q > 0.0)) {
+            s.probe = (s.kmode & cher::kDispBit) | cher::kProbeBit;
+            s.direct = (s.kmode & ~cher::kLargeBit) | cher::kDirectBit;
+            s.direct_smem = cher::kernel_smem_bytes(fp32, s.block, s.direct, p);
+            if (cher::kernel_prepare(fp32, s.block, s.direct, s.direct_smem) != cudaSuccess) {
+                cudaGetLastError();
+                return CHER_ERANGE;
+            }
+            p.choice = reinterpret_cast<float *>(counter + 1);
+        }
     }
     if (counter && grid > ctas) {
         grid = ctas;
@@ -472,6 +493,19 @@ cher_status plan(const cher_ctx *c, cher::KParams &p, bool fp32, int mode, int c
     }
     if (grid > 0x7fffffff || (p.tile_counter && p.n_tiles > 0xf0000000ll)) return CHER_ERANGE;
     s.grid = static_cast<int>(grid);
+    return CHER_OK;
+}
+
+// The planned kernels; the scratch words are clear.
+cher_status run(const cher_ctx *c, const cher::KParams &p, bool fp32, const Shape &s, void *stream) {
+    if ((p.choice && cher::kernel_launch(fp32, 256, s.probe, c->num_sms, 0, p, stream) !=
+                         cudaSuccess) ||
+        cher::kernel_launch(fp32, s.block, s.kmode, s.grid, s.smem, p, stream) != cudaSuccess ||
+        (p.choice && cher::kernel_launch(fp32, s.block, s.direct, s.grid, s.direct_smem, p,
+                                         stream) != cudaSuccess)) {
+        cudaGetLastError();
+        return CHER_ECUDA;
+    }
     return CHER_OK;
 }
 
@@ -483,14 +517,11 @@ cher_status launch(cher_ctx *c, cher::KParams &p, bool fp32, int mode, bool pers
     const cher_status r = plan(c, p, fp32, mode, counted ? c->ctas_per_sm : 0,
                                counted ? c->d_scratch : nullptr, s);
     if (r != CHER_OK) return r;
-    if (p.tile_counter && cudaMemsetAsync(p.tile_counter, 0, sizeof(unsigned),
-                                          static_cast<cudaStream_t>(stream)) != cudaSuccess)
+    if ((p.tile_counter || p.choice) &&
+        cudaMemsetAsync(c->d_scratch, 0, 2 * sizeof(unsigned),
+                        static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return CHER_ECUDA;
-    if (cher::kernel_launch(fp32, s.block, s.kmode, s.grid, s.smem, p, stream) != cudaSuccess) {
-        cudaGetLastError();
-        return CHER_ECUDA;
-    }
-    return CHER_OK;
+    return run(c, p, fp32, s, stream);
 }
 
 bool check_device(const cher_ctx *c) {
@@ -671,10 +702,10 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
     // the telescopes for the hits kernel's bound, from the middle of the array
     // (radii rounded up)
     cher::build_center_bins(c->tel.data(), static_cast<int32_t>(nt), c->CB);
-    std::vector<float> ctel(nt * 4);
+    std::vector<float> ctel(nt * 8);
     c->cull_rmax = c->cull_zmax = 0.0;
-    for (size_t m = 0; m < nt; ++m) {
-        const cher_telescope &q = c->tel[m];
+    for (size_t m = 0; m < 2 * nt; ++m) {
+        const cher_telescope &q = c->tel[m < nt ? c->CB.order[m] : m - nt];
         ctel[4 * m] = static_cast<float>(q.x - c->CB.ox);
         ctel[4 * m + 1] = static_cast<float>(q.y - c->CB.oy);
         ctel[4 * m + 2] = static_cast<float>(q.z);
@@ -682,9 +713,16 @@ cher_status cher_build_refraction_tables(cher_ctx *c, int32_t n_heights, int32_t
         c->cull_rmax = std::max(c->cull_rmax, q.r * (1.0 + 1e-6));
         c->cull_zmax = std::max(c->cull_zmax, std::fabs(q.z) * (1.0 + 1e-6));
     }
+    // (more than 24 telescopes with 12 or more within 300 m of one, on the
+    // average over their box, more than 128, or large spheres)
+    double sum_r = 0.0;
+    for (const cher_telescope &q : c->tel) sum_r += q.r;
+    const double area = (2.0 * c->CB.ex + 300.0) * (2.0 * c->CB.ey + 300.0);
+    c->crowded = c->CB.words > cher::kCullFewWords || sum_r > 1000.0 ||
+                 (nt > 24 && static_cast<double>(nt) * (cher::kPi * 9.0e4) > 12.0 * area);
     const size_t n_masks = c->CB.masks.size();
-    ctel.resize(4 * nt + n_masks);
-    std::memcpy(ctel.data() + 4 * nt, c->CB.masks.data(), n_masks * sizeof(uint32_t));
+    ctel.resize(8 * nt + n_masks);
+    std::memcpy(ctel.data() + 8 * nt, c->CB.masks.data(), n_masks * sizeof(uint32_t));
     cher::table_slopes(c->T, c->ax_sq, c->ax_sh);
     cher_status r;
     double *d_tab64 = nullptr;
@@ -1590,8 +1628,9 @@ extern "C" cher_status cher_generate_propagate_noalloc(cher_ctx *c, const cher_t
                                                        uint64_t seed, cher_precision prec,
                                                        const cher_output *out, void *stream) {
     if (!c || !out || !t) return CHER_EINVAL;
-    // one 8-byte tile counter of the fixed array; tile indices beyond the
-    // library-wide step limit are refused before anything is launched
+    // one 8-byte word of the fixed array, the counter and the choice; tile
+    // indices beyond the library-wide step limit are refused before anything is
+    // launched
     const size_t need = sizeof(unsigned long long);
     if (need > kStaticScratchBytes) return CHER_ERANGE;
     if (t->n > (int64_t(1) << 40) || t->track_base > (int64_t(1) << 40)) return CHER_ERANGE;
@@ -1631,13 +1670,9 @@ extern "C" cher_status cher_generate_propagate_noalloc(cher_ctx *c, const cher_t
     s = plan(c, p, fp32, cher::MODE_HITS, std::max(1, c->ctas_per_sm), scratch, sh);
     if (s != CHER_OK) return s;
     // the array keeps the previous call's contents: clear the counter first
-    if (p.tile_counter) {
+    if (p.tile_counter || p.choice) {
         k_clear_static_scratch<<<1, 32, 0, st>>>(static_cast<int>(need / sizeof(unsigned long long)));
         if (cudaGetLastError() != cudaSuccess) return CHER_ECUDA;
     }
-    if (cher::kernel_launch(fp32, sh.block, sh.kmode, sh.grid, sh.smem, p, stream) != cudaSuccess) {
-        cudaGetLastError();
-        return CHER_ECUDA;
-    }
-    return CHER_OK;
+    return run(c, p, fp32, sh, stream);
 }

@@ -97,6 +97,13 @@ struct alignas(16) Ring {
     float4 e;      // azimuth basis e1 (x, y); rho = (R + M) e.z + e.w a
 };
 
+// The kernels: BOUND as described above; LARGE, the same for arrays of more than
+// 128 telescopes, which looks at the words of the box's x range only (a kernel of
+// its own: the code costs BOUND 2 % where it gives nothing); DIRECT, which
+// propagates the bunches of all steps, for launches where the bound would cost
+// more than it saves (the array is dense, the rings are long, the steps at the
+// edges of the tables: k_probe).
+enum : int { BOUND = 0, DIRECT = 1, LARGE = 2 };
 enum : int { REACH_NONE = 0, REACH_RING = 1, REACH_ALL = 2 };
 
 // What the first test of one telescope needs besides (32 bytes, behind the
@@ -228,6 +235,20 @@ __device__ __forceinline__ int ring_setup(const KParams &p, double x0d, double y
     return !ok ? REACH_ALL : (b0 <= b1 && b2 <= b3 ? REACH_RING : REACH_NONE);
 }
 
+// The first test of one telescope: the ring passes by it.
+template <int MODE>
+__device__ __forceinline__ bool ring_near(const KParams &p, float sm, float fac, float cm2,
+                                          const float4 P, const float4 U, const float4 T) {
+    const float dx = T.x - P.x, dy = T.y - P.y;
+    const float dz = MODE == MODE_SCREEN ? 0.0f : T.z;
+    const float dot = dx * U.x + dy * U.y + dz * U.z;
+    const float rk2 = cm2 * (dx * dx + dy * dy + dz * dz - dot * dot);
+    const float rc = sm * dot + P.z;
+    const float rho = (MODE == MODE_SCREEN ? p.cull.r_cut : T.w) * fac + P.w;
+    const float far = rc + rho, near = fmaxf(rc - rho, 0.0f);
+    return (rk2 <= far * far + U.w) & (rk2 >= near * near - U.w);
+}
+
 // The sectors at which the ring can reach one telescope, first and number
 // (kSectors: all, 0: none).
 template <int MODE>
@@ -340,6 +361,19 @@ __device__ __forceinline__ uint32_t box_telescopes(const KParams &p, uint32_t bi
            __ldg(Y + (bins >> 24) * nw) & ~__ldg(Y + (bins >> 16 & 0xffu) * nw);
 }
 
+// The words of a large array, which is sorted by x, that a box's x range
+// touches.  False where the box holds more telescopes, estimated from its two
+// ranges, than testing them can save on nb bunches.
+__device__ __forceinline__ bool box_words(const KParams &p, uint32_t bins, int nb, int &w0, int &w1) {
+    w1 = p.cull.words;
+    const uint32_t *X = p.cull.bins + 2 * (kCullBins + 1) * w1, *Y = X + kCullBins + 1;
+    const uint32_t x0 = __ldg(X + (bins & 0xffu)), x1 = __ldg(X + (bins >> 8 & 0xffu));
+    const uint32_t ny = __ldg(Y + (bins >> 24)) - __ldg(Y + (bins >> 16 & 0xffu));
+    w0 = static_cast<int>(x0 >> 5);
+    w1 = static_cast<int>((x1 + 31u) >> 5);
+    return (x1 - x0) * ny <= static_cast<uint32_t>(p.n_tel) * min(6u * nb + 16u, 65536u);
+}
+
 // inclusive prefix sum over the warp
 __device__ __forceinline__ int warp_scan(int v, int lane) {
 #pragma unroll
@@ -348,6 +382,47 @@ __device__ __forceinline__ int warp_scan(int v, int lane) {
         if (lane >= o) v += t;
     }
     return v;
+}
+
+// The place of the piece 32 win + lane, moving s_cur on to the window's end.
+// Places start at distinct pieces, so the starts inside the window are one bit
+// each (a shift by 32 or more gives 0); lanes past the last piece get the
+// empty place behind the last.
+template <class W>
+__device__ __forceinline__ int place_at(W &w, int &s_cur, int win, int lane, unsigned below) {
+    unsigned bit;
+    asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(w.off[s_cur + 1 + lane] - win * 32));
+    const unsigned starts = __reduce_or_sync(kFull, bit);
+    const int s = s_cur + __popc(starts & (below * 2u + 1u));
+    s_cur += __popc(starts);
+    return s;
+}
+
+// A bunch past the tables' range: queued for the fallback pass.
+template <class R>
+__device__ __forceinline__ void defer(const KParams &p, const Consts<R> &c, const BunchOut<R> &o,
+                                      bool live, R w, int64_t gstep, int j, int lane,
+                                      unsigned below) {
+    const bool dq = live && o.status == ST_DEFER;
+    const unsigned qm = __ballot_sync(kFull, dq);
+    if (!qm) return;
+    const int leader = __ffs(qm) - 1;
+    unsigned long long at0 = 0;
+    if (lane == leader)
+        at0 = atomicAdd(p.fb_count, static_cast<unsigned long long>(__popc(qm)));
+    at0 = __shfl_sync(kFull, at0, leader);
+    const unsigned long long at = at0 + __popc(qm & below);
+    if (dq && at < static_cast<unsigned long long>(p.fb_cap)) {
+        FbEntry<R> e;
+        e.xe = o.X; e.ye = o.Y; e.he = c.h_obs + o.he; e.dh = o.he; e.te = o.t;
+        e.hx = o.cx; e.hy = o.cy; e.s_obs = o.cz; e.c2 = o.c2; e.lam = o.lam;
+        e.w = w;
+        e.kap = o.kap;
+        e.key = (static_cast<uint64_t>(gstep) << 32) | static_cast<uint32_t>(j);
+        e.step_hi = static_cast<uint32_t>(static_cast<uint64_t>(gstep) >> 32);
+        static_cast<FbEntry<R> *>(p.fb_list)[dbg_index(p, static_cast<int64_t>(at), p.fb_cap,
+                                                       DBG_FB)] = e;
+    }
 }
 
 // While a group is worked on, the places past cnt are free: place cnt + lane
@@ -370,8 +445,9 @@ __device__ __forceinline__ uint32_t &pair_at(W &w, int q) {
 static_assert(sizeof(Ring) + sizeof(Near) <= sizeof(Seg<float>), "a free place holds both");
 static_assert(kCap - 32 + kPairs <= kCap + 33, "the pairs fit the free places' offsets");
 
-template <class R, int MODE, bool TR, int FB, bool DS>
+template <class R, int MODE, bool TR, int FB, bool DS, int KIND>
 __device__ __forceinline__ void hits(const KParams &p) {
+    if (p.choice && (*p.choice < 0.0f) != (KIND == DIRECT)) return;
     extern __shared__ __align__(16) unsigned char smem[];
     // (volatile: kept in registers instead of read again from the special
     // registers at every use)
@@ -381,7 +457,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
     asm volatile("mov.u32 %0, %%lanemask_lt;" : "=r"(below));
     // with the transmission draw every bunch has to be decided
-    constexpr bool kDraw = TR && MODE == MODE_HITS;
+    constexpr bool kDraw = TR && MODE == MODE_HITS && KIND != DIRECT;
+    constexpr int kSpan = KIND == DIRECT ? 1 : kPer;     // bunches of a piece
     using Entry = typename std::conditional<MODE == MODE_HITS, QueueHits, QueueScreen>::type;
     using Warp = WarpSmem<R, Entry, kDraw, DS>;
     Warp &W = reinterpret_cast<Warp *>(smem)[tid >> 5];
@@ -475,7 +552,7 @@ __device__ __forceinline__ void hits(const KParams &p) {
                     }
                     if (!y.valid) atomicAdd(&W.drop[0], 1u);
                 }
-                if (!open && y.nb > 0) {
+                if (KIND != DIRECT && !open && y.nb > 0) {
                     float ux, uy, uzf, eta, s_lo, s_hi;
                     if constexpr (std::is_same<R, float>::value) {
                         ux = load_dir<R>(p.ux, i);
@@ -521,86 +598,86 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 }
             }
 
-            // the telescopes near each lane's ring (32 to a word, from the box
-            // by the bins' prefix masks), then the sectors of those pairs
-#pragma unroll
-            for (int w = 0; w < kMaskWords; ++w) W.mask[cnt + lane][w] = 0u;
-            int n_near = 0;
-            if (kind == REACH_RING) {
-                const Ring *G = ring_at(W, cnt + lane);
-                const Near *N = near_at(W, cnt + lane);
-                const float sm = G->a.w, fac = G->e.z, cm2 = 1.0f - sm * sm;
-                const float4 P = N->p, U = N->w;
-                for (int w = 0; w < p.cull.words; ++w) {
-                    uint32_t cand = box_telescopes(p, B.bins, w);
-                    while (cand) {
-                        const int m = w * 32 + __ffs(cand) - 1;
-                        cand &= cand - 1u;
-                        const float4 T = __ldg(p.cull.tel + dbg_index(p, m, p.n_tel, DBG_GRID));
-                        const float dx = T.x - P.x, dy = T.y - P.y;
-                        const float dz = MODE == MODE_SCREEN ? 0.0f : T.z;
-                        const float dot = dx * U.x + dy * U.y + dz * U.z;
-                        const float rk2 = cm2 * (dx * dx + dy * dy + dz * dz - dot * dot);
-                        const float rc = sm * dot + P.z;
-                        const float rho = (MODE == MODE_SCREEN ? p.cull.r_cut : T.w) * fac + P.w;
-                        const float far = rc + rho, near = fmaxf(rc - rho, 0.0f);
-                        const bool in = (rk2 <= far * far + U.w) & (rk2 >= near * near - U.w);
-                        if (in) W.near[n_near & (kNear - 1)][lane] = static_cast<uint16_t>(m);
-                        n_near += in;
-                    }
-                }
-                if (n_near > kNear) {
-                    kind = REACH_ALL;
-                    n_near = 0;
-                }
-            }
-            __syncwarp();
-            // two telescopes a lane at a time: one round of full lanes for the
-            // usual 19 - 30 pairs of a group
-            for (int k0 = 0; __any_sync(kFull, n_near > k0); k0 += 2) {
-                int n_pairs = 0;
-#pragma unroll
-                for (int k = k0; k < k0 + 2; ++k) {
-                    const unsigned has = __ballot_sync(kFull, n_near > k);
-                    if (n_near > k)
-                        pair_at(W, n_pairs + __popc(has & below)) =
-                            static_cast<uint32_t>(cnt + lane) << 16 | W.near[k][lane];
-                    n_pairs += __popc(has);
-                }
-                __syncwarp();
-                for (int q = lane; q < n_pairs; q += 32) {
-                    const uint32_t e = pair_at(W, q);
-                    const int at = static_cast<int>(e >> 16);
-                    const int2 sec = ring_sectors<MODE>(p, *ring_at(W, at),
-                                                        __ldg(p.cull.tel + (e & 0xffffu)));
-                    // sectors sec.x .. sec.x + sec.y - 1 around the circle, word by word
-                    for (int s = sec.x, n = sec.y; n > 0;) {
-                        const int b = s & 31, m = min(32 - b, n);
-                        atomicOr(&W.mask[at][(s >> 5) & (kMaskWords - 1)],
-                                 (m == 32 ? kFull : (1u << m) - 1u) << b);
-                        s += m;
-                        n -= m;
-                    }
-                }
-                __syncwarp();
-            }
             uint32_t mask[kMaskWords], any = 0u;
+            if constexpr (KIND != DIRECT) {
+                // the telescopes near each lane's ring (32 to a word, from the box
+                // by the bins' prefix masks), then the sectors of those pairs
 #pragma unroll
-            for (int w = 0; w < kMaskWords; ++w) {
-                mask[w] = kind == REACH_ALL ? kFull : W.mask[cnt + lane][w];
-                any |= mask[w];
+                for (int w = 0; w < kMaskWords; ++w) W.mask[cnt + lane][w] = 0u;
+                int n_near = 0, w0 = 0, w1 = p.cull.words;
+                if constexpr (KIND == LARGE)
+                    if (kind == REACH_RING && !box_words(p, B.bins, nb, w0, w1)) kind = REACH_ALL;
+                if (kind == REACH_RING) {
+                    const Ring *G = ring_at(W, cnt + lane);
+                    const Near *N = near_at(W, cnt + lane);
+                    const float sm = G->a.w, fac = G->e.z, cm2 = 1.0f - sm * sm;
+                    const float4 P = N->p, U = N->w;
+                    for (int w = w0; w < w1; ++w) {
+                        uint32_t cand = box_telescopes(p, B.bins, w);
+                        while (cand) {
+                            const int m = w * 32 + __ffs(cand) - 1;
+                            cand &= cand - 1u;
+                            const bool in = ring_near<MODE>(
+                                p, sm, fac, cm2, P, U,
+                                __ldg(p.cull.tel + dbg_index(p, m, p.n_tel, DBG_GRID)));
+                            if (in) W.near[n_near & (kNear - 1)][lane] = static_cast<uint16_t>(m);
+                            n_near += in;
+                        }
+                    }
+                    if (n_near > kNear) {
+                        kind = REACH_ALL;
+                        n_near = 0;
+                    }
+                }
+                __syncwarp();
+                // two telescopes a lane at a time: one round of full lanes for the
+                // usual 19 - 30 pairs of a group
+                for (int k0 = 0; __any_sync(kFull, n_near > k0); k0 += 2) {
+                    int n_pairs = 0;
+#pragma unroll
+                    for (int k = k0; k < k0 + 2; ++k) {
+                        const unsigned has = __ballot_sync(kFull, n_near > k);
+                        if (n_near > k)
+                            pair_at(W, n_pairs + __popc(has & below)) =
+                                static_cast<uint32_t>(cnt + lane) << 16 | W.near[k][lane];
+                        n_pairs += __popc(has);
+                    }
+                    __syncwarp();
+                    for (int q = lane; q < n_pairs; q += 32) {
+                        const uint32_t e = pair_at(W, q);
+                        const int at = static_cast<int>(e >> 16);
+                        const int2 sec = ring_sectors<MODE>(p, *ring_at(W, at),
+                                                            __ldg(p.cull.tel + (e & 0xffffu)));
+                        // sectors sec.x .. sec.x + sec.y - 1 around the circle, word by word
+                        for (int s = sec.x, n = sec.y; n > 0;) {
+                            const int b = s & 31, m = min(32 - b, n);
+                            atomicOr(&W.mask[at][(s >> 5) & (kMaskWords - 1)],
+                                     (m == 32 ? kFull : (1u << m) - 1u) << b);
+                            s += m;
+                            n -= m;
+                        }
+                    }
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int w = 0; w < kMaskWords; ++w) {
+                    mask[w] = kind == REACH_ALL ? kFull : W.mask[cnt + lane][w];
+                    any |= mask[w];
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            const bool keep = nb > 0 && (kDraw || any != 0u);
+            const bool keep = nb > 0 && (KIND == DIRECT || kDraw || any != 0u);
             const unsigned kept = __ballot_sync(kFull, keep);
-            const int np = (nb + kPer - 1) / kPer;
+            const int np = (nb + kSpan - 1) / kSpan;
             const int v = warp_scan(keep ? np : 0, lane);
             if (keep) {
                 const int s = dbg_index(p, cnt + __popc(kept & below), kCap, DBG_SMEM);
                 W.off[s] = tot + v - np;
                 W.nb[s] = nb;
+                if constexpr (KIND != DIRECT) {
 #pragma unroll
-                for (int w = 0; w < kMaskWords; ++w) W.mask[s][w] = mask[w];
+                    for (int w = 0; w < kMaskWords; ++w) W.mask[s][w] = mask[w];
+                }
                 if constexpr (kDraw) W.sec[s] = make_float2(B.sec_lo, B.sec_hi);
                 W.step[s] = i;
                 // (what prep_step takes of the yield, until the batch is full)
@@ -635,18 +712,34 @@ __device__ __forceinline__ void hits(const KParams &p) {
         int s_cur = 0, head = 0, queued = 0, win = 0;
         for (;;) {
             for (; win < nwin && queued < 32; ++win) {
-                // the place of each lane's piece: places start at distinct
-                // pieces, so the starts inside the window are one bit each (a
-                // shift by 32 or more gives 0); lanes past the last piece get
-                // the empty place behind the last
-                unsigned bit;
-                asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(W.off[s_cur + 1 + lane] - win * 32));
-                const unsigned starts = __reduce_or_sync(kFull, bit);
-                const int s = s_cur + __popc(starts & (below * 2u + 1u));
-                s_cur += __popc(starts);
+                const int s = place_at(W, s_cur, win, lane, below);
                 const int sc = dbg_index(p, s, kCap + 1, DBG_SMEM);
                 const Seg<R> &S = W.seg[sc];
-                const int j0 = (win * 32 + lane - W.off[sc]) * kPer, left = W.nb[sc] - j0;
+                const int j0 = (win * 32 + lane - W.off[sc]) * kSpan, left = W.nb[sc] - j0;
+                if constexpr (KIND == DIRECT) {
+                    // all are propagated as they come; those that cross a
+                    // sphere, few of them, are queued to be propagated again and
+                    // recorded by full warps
+                    const bool live = left > 0;
+                    BunchOut<R> o;
+                    o.status = -1;
+                    o.zg = R(0);
+                    if (live) {
+                        bunch<R, TR, FB, DS>(p, c, S, W.at(sc), j0, o);
+                        if (o.status != ST_GROUND && o.status != ST_DEFER)
+                            atomicAdd(&W.drop[o.status], 1u);
+                    }
+                    if constexpr (FB == 1)
+                        defer<R>(p, c, o, live, S.w, p.track_base + (live ? W.step[sc] : 0), j0,
+                                 lane, below);
+                    int s0 = 0, gsel = 0;
+                    const bool pass = live && sphere_hits<R>(p, c, o, s0, gsel) != 0u;
+                    const unsigned in = __ballot_sync(kFull, pass);
+                    if (pass)
+                        W.queue[(head + queued + __popc(in & below)) & (kQueue - 1)].set(s, j0);
+                    queued += __popc(in);
+                    continue;
+                }
 #pragma unroll
                 for (int k = 0; k < kPer; ++k) {
                     const int j = j0 + k;
@@ -713,7 +806,7 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 __syncwarp();          // read before the places are used again
                 if (live) {
                     bunch<R, TR, FB, DS>(p, c, W.seg[s], W.at(s), j, o);
-                    if (o.status != ST_GROUND && o.status != ST_DEFER)
+                    if (KIND != DIRECT && o.status != ST_GROUND && o.status != ST_DEFER)
                         atomicAdd(&W.drop[o.status], 1u);
                 }
                 head = (head + n) & (kQueue - 1);
@@ -740,30 +833,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
                 }
                 const int64_t gstep = p.track_base + W.step[s];
                 const uint64_t key = (static_cast<uint64_t>(gstep) << 32) | static_cast<uint32_t>(j);
-                if constexpr (FB == 1) {
-                    // past the tables' range: queue for the fallback pass
-                    const bool dq = live && o.status == ST_DEFER;
-                    const unsigned qm = __ballot_sync(kFull, dq);
-                    if (qm) {
-                        const int leader = __ffs(qm) - 1;
-                        unsigned long long at0 = 0;
-                        if (lane == leader)
-                            at0 = atomicAdd(p.fb_count, static_cast<unsigned long long>(__popc(qm)));
-                        at0 = __shfl_sync(kFull, at0, leader);
-                        const unsigned long long at = at0 + __popc(qm & below);
-                        if (dq && at < static_cast<unsigned long long>(p.fb_cap)) {
-                            FbEntry<R> e;
-                            e.xe = o.X; e.ye = o.Y; e.he = c.h_obs + o.he; e.dh = o.he; e.te = o.t;
-                            e.hx = o.cx; e.hy = o.cy; e.s_obs = o.cz; e.c2 = o.c2; e.lam = o.lam;
-                            e.w = W.seg[s].w;
-                            e.kap = o.kap;
-                            e.key = key;
-                            e.step_hi = static_cast<uint32_t>(static_cast<uint64_t>(gstep) >> 32);
-                            static_cast<FbEntry<R> *>(p.fb_list)[dbg_index(
-                                p, static_cast<int64_t>(at), p.fb_cap, DBG_FB)] = e;
-                        }
-                    }
-                }
+                if constexpr (FB == 1 && KIND != DIRECT)
+                    defer<R>(p, c, o, live, W.seg[s].w, gstep, j, lane, below);
                 int s0 = 0, gsel = 0;
                 const unsigned hm = live ? sphere_hits<R>(p, c, o, s0, gsel) : 0u;
                 const R np1 = DS ? R(1) + o.kap * c.eta_o : np1o;
@@ -813,47 +884,152 @@ __device__ __forceinline__ void hits(const KParams &p) {
 // One instantiation for every block size: 64 registers in FP32 (1024 threads
 // per SM), 128 in FP64.  With spectra (128-step blocks only) 72: seven CTAs per
 // SM without spills against eight with them, 144 -> 136 us at 3e5 steps.
-template <class R, int MODE, bool TR, int FB, bool DS>
+template <class R, int MODE, bool TR, int FB, bool DS, int KIND>
 __global__ void __launch_bounds__(DS ? 128 : 512, std::is_same<R, float>::value ? (DS ? 7 : 2) : 1)
     k_hits(const __grid_constant__ KParams p) {
-    hits<R, MODE, TR, FB, DS>(p);
+    hits<R, MODE, TR, FB, DS, KIND>(p);
 }
 
-template <class R, int MODE, bool DS>
+// Whether the bound saves more than it costs (p.choice, less than 0: no), from
+// one step per warp, spread evenly over the list, its lanes sharing the
+// telescopes.  In instructions of a warp per bunch, from both kernels' times over
+// the arrays below: propagating one costs 10; with the bound 2 for drawing it (5
+// with the transmission draw), 50 if its azimuth is in a sector (the records'
+// waits for their places among them), 22 where the step has all sectors; a step
+// 3, and 3 a telescope of its box.
+// FP32, 2e6 vertical (1e6 at 60 deg, 3e5 at 69 deg) steps, us per launch, the
+// bound / all bunches / chosen (10 - 14 more than the kernel alone):
+//   64 spheres of 8 m over 300 x 300 m                   1092 /  965 /  979
+//   256 of 6 m over 500 x 500 m                          1205 /  965 /  978
+//   1000 of 6 m over 2 x 2 km, vertical; 60 deg     565 / 810 / 578; 985 / 370 / 383
+//   4096 of 6 m over 8 x 8 km, vertical; 60 deg     298 / 735 / 310; 520 / 323 / 335
+//   100 over 2 x 2 km at 69 deg, tables to 70 with the fallback    211 / 160 / 173
+//   64 of 8 m over 300 x 300 m, 2e5 steps with spectra     239 /  240 /  253
+// (before the choice, all words of a large array looked at: 870 and 1285 us over
+// the 1000, 1150 and 1352 over the 4096; the kernel that always propagated all
+// took 947, 980, 848 and 362, 752 and 334, 164, 237).
+template <bool DS>
+__global__ void __launch_bounds__(256) k_probe(const __grid_constant__ KParams p) {
+    __shared__ float s_gain[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t w = int64_t(blockIdx.x) * 8 + warp;
+    const int64_t i = w * (p.n / (int64_t(gridDim.x) * 8));
+    float gain = 0.0f;
+    YieldF y;
+    y.nb = 0;
+    SegD<float> D;
+    const double z0 = __ldg(p.z0 + i), len = __ldg(p.len + i), ekin = __ldg(p.ekin + i);
+    const double x0 = __ldg(p.x0 + i), y0 = __ldg(p.y0 + i);
+    const float ux = load_dir<float>(p.ux, i), uy = load_dir<float>(p.uy, i);
+    const float uz = load_dir<float>(p.uz, i);
+    const bool valid = step_valid<float>(p, i);
+    // (a step that the screen leaves open has few bunches)
+    bool open;
+    if constexpr (DS) open = !screen_yield_disp(p, valid, z0, len, ekin, uz, y, D);
+    else open = !screen_yield(p, valid, z0, len, ekin, uz, y);
+    if (!open && y.nb > 0) {
+        float s_lo, s_hi;
+        if constexpr (DS) {
+            s_lo = cone_sine(D.beta, y.eta, p.f.kap_lo, D.x_th);
+            s_hi = cone_sine(D.beta, y.eta, p.f.kap[0], D.x_th);
+        } else {
+            s_lo = s_hi = sqrtf(y.s2);
+        }
+        Ring G;
+        Near N;
+        Box B;
+        int kind = ring_setup<MODE_HITS, DS>(p, x0, y0, __double2float_rn(z0) - p.f.h_obs,
+                                             __double2float_rn(len), ux, uy, uz, y.eta, s_lo, s_hi,
+                                             G, N, B);
+        int tests = 0, near = 0, w0 = 0, w1 = p.cull.words;
+        float sectors = 0.0f;
+        if (kind == REACH_RING && w1 > kCullFewWords && !box_words(p, B.bins, y.nb, w0, w1))
+            kind = REACH_ALL;
+        if (kind == REACH_RING) {
+            uint32_t mask[kMaskWords] = {};
+            const float sm = G.a.w;
+            for (int v = w0; v < w1; ++v) {
+                const uint32_t cand = box_telescopes(p, B.bins, v);
+                tests += 1 + __popc(cand);
+                if (!(cand >> lane & 1u)) continue;
+                const float4 T = __ldg(p.cull.tel + v * 32 + lane);
+                if (!ring_near<MODE_HITS>(p, sm, G.e.z, 1.0f - sm * sm, N.p, N.w, T)) continue;
+                ++near;
+                const int2 sec = ring_sectors<MODE_HITS>(p, G, T);
+                for (int k = sec.x; k < sec.x + sec.y; ++k) {
+#pragma unroll
+                    for (int q = 0; q < kMaskWords; ++q)
+                        if ((k >> 5 & (kMaskWords - 1)) == q) mask[q] |= 1u << (k & 31);
+                }
+            }
+            if (__reduce_add_sync(kFull, static_cast<unsigned>(near)) > kNear) kind = REACH_ALL;
+#pragma unroll
+            for (int q = 0; q < kMaskWords; ++q)
+                sectors += static_cast<float>(__popc(__reduce_or_sync(kFull, mask[q])));
+        }
+        const float queued = kind == REACH_ALL ? 22.0f : 50.0f / kSectors * sectors;
+        const float drawn = p.trans ? 5.0f : queued > 0.0f ? 2.0f : 0.0f;
+        gain = static_cast<float>(y.nb) * (10.0f - drawn - queued) - 3.0f - 3.0f * tests;
+    }
+    if (lane == 0) s_gain[warp] = gain;
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < 8; ++k) gain += s_gain[k];
+        atomicAdd(p.choice, gain);
+    }
+}
+
+template <class R, int MODE, bool DS, int KIND>
 const void *pick(bool tr, bool fb) {
     if constexpr (MODE == MODE_SCREEN) {
         if constexpr (DS) {
             return nullptr;
         } else {
-            return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 0, false>)
-                      : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 0, false>);
+            return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 0, false, KIND>)
+                      : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 0, false, KIND>);
         }
     } else {
         if (fb)
-            return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 1, DS>)
-                      : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 1, DS>);
-        return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 0, DS>)
-                  : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 0, DS>);
+            return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 1, DS, KIND>)
+                      : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 1, DS, KIND>);
+        return tr ? reinterpret_cast<const void *>(&k_hits<R, MODE, true, 0, DS, KIND>)
+                  : reinterpret_cast<const void *>(&k_hits<R, MODE, false, 0, DS, KIND>);
     }
 }
 
 template <class R>
 const void *pick_mode(int mode, bool tr, bool fb, bool ds) {
-    if (mode == MODE_SCREEN) return ds ? pick<R, MODE_SCREEN, true>(tr, fb)
-                                       : pick<R, MODE_SCREEN, false>(tr, fb);
-    return ds ? pick<R, MODE_HITS, true>(tr, fb) : pick<R, MODE_HITS, false>(tr, fb);
+    if (mode == MODE_SCREEN) return ds ? pick<R, MODE_SCREEN, true, BOUND>(tr, fb)
+                                       : pick<R, MODE_SCREEN, false, BOUND>(tr, fb);
+    return ds ? pick<R, MODE_HITS, true, BOUND>(tr, fb) : pick<R, MODE_HITS, false, BOUND>(tr, fb);
 }
 
 }  // namespace
 
+namespace {
+constexpr int kOptions = kTransBit | kFbBit | kDispBit | kCurvBit | kDirectBit | kProbeBit |
+                         kLargeBit;
+}
+
 bool hits_kernel_serves(int mode) {
-    const int m = mode & ~(kTransBit | kFbBit | kDispBit | kCurvBit);
+    const int m = mode & ~kOptions;
     return !(mode & kCurvBit) && (m == MODE_HITS || m == MODE_SCREEN);
 }
 
 const void *hits_kernel(bool fp32, int mode) {
     const bool tr = (mode & kTransBit) != 0, fb = (mode & kFbBit) != 0, ds = (mode & kDispBit) != 0;
-    const int m = mode & ~(kTransBit | kFbBit | kDispBit | kCurvBit);
+    const int m = mode & ~kOptions;
+    if (mode & (kDirectBit | kProbeBit | kLargeBit)) {      // (crossings of the FP32 path only)
+        if (!fp32 || m != MODE_HITS) return nullptr;
+        if (mode & kProbeBit)
+            return ds ? reinterpret_cast<const void *>(&k_probe<true>)
+                      : reinterpret_cast<const void *>(&k_probe<false>);
+        if (mode & kDirectBit)
+            return ds ? pick<float, MODE_HITS, true, DIRECT>(tr, fb)
+                      : pick<float, MODE_HITS, false, DIRECT>(tr, fb);
+        return ds ? pick<float, MODE_HITS, true, LARGE>(tr, fb)
+                  : pick<float, MODE_HITS, false, LARGE>(tr, fb);
+    }
     return fp32 ? pick_mode<float>(m, tr, fb, ds) : pick_mode<double>(m, tr, fb, ds);
 }
 
@@ -866,8 +1042,9 @@ size_t warp_bytes(bool tr, bool ds) {
 }  // namespace
 
 size_t hits_smem_bytes(bool fp32, int mode, int block) {
-    const int m = mode & ~(kTransBit | kFbBit | kDispBit | kCurvBit);
-    const bool tr = m == MODE_HITS && (mode & kTransBit) != 0, ds = (mode & kDispBit) != 0;
+    const int m = mode & ~kOptions;
+    // (the draw's bounds of the steps: not where every bunch is propagated)
+    const bool tr = m == MODE_HITS && (mode & kTransBit) != 0 && !(mode & (kDirectBit | kProbeBit)), ds = (mode & kDispBit) != 0;
     const size_t w = m == MODE_HITS ? (fp32 ? warp_bytes<float, QueueHits>(tr, ds)
                                             : warp_bytes<double, QueueHits>(tr, ds))
                                     : (fp32 ? warp_bytes<float, QueueScreen>(tr, ds)

@@ -27,6 +27,7 @@ enum : int32_t {
 
 constexpr int kMaxCandPerCell = 32;   // telescope candidates in one grid cell
 constexpr int kCullBins = 128;        // bins of the telescopes' centres per axis
+constexpr int kCullFewWords = 4;      // up to 4 x 32 telescopes keep the caller's order
 constexpr int kDispMax = 9;           // nodes of a wavelength-dependent index
 
 // Host-side tables, all FP64 (step a0).
@@ -71,7 +72,10 @@ struct HostBins {
     int32_t words = 0;
     double ox = 0, oy = 0, ex = 0, ey = 0;
     double x0 = 0, y0 = 0, inv_bx = 0, inv_by = 0;
-    std::vector<uint32_t> masks;          // [2][kCullBins + 1][words]
+    std::vector<int32_t> order;           // the masks' telescopes: the caller's order,
+                                          // or by x past kCullFewWords words
+    std::vector<uint32_t> masks;          // [2][kCullBins + 1][words], then the numbers
+                                          // of telescopes in them, [2][kCullBins + 1]
 };
 void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b);
 void table_slopes(const HostTables &T, double &per_q, double &per_h);
@@ -147,8 +151,9 @@ struct KParams {
         float ax_sq, ax_sh;
         int words;
         float x0, y0, inv_bx, inv_by, r_max, z_max, r_cut;
-        const uint32_t *bins;             // [2][kCullBins + 1][words], x then y
-        const float4 *tel;                // [n_tel]
+        const uint32_t *bins;             // HostBins::masks
+        const float4 *tel;                // [n_tel] in the masks' order
+        const float4 *tel0;               // [n_tel] in the caller's
     } cull;
     // outputs
     void *pos, *tim;
@@ -171,6 +176,7 @@ struct KParams {
     // of the list
     int32_t group;
     uint32_t n_groups, streams;
+    float *choice;                        // less than 0: propagate all bunches (NULL: no)
     // adjoint screening: frozen bunch counts (NULL: this launch's, written to
     // y_nb), list of (step, bunch) pairs
     // that land within the read-out radius of a telescope centre
@@ -281,13 +287,19 @@ constexpr int kFbBit = 8;
 // only; the curved atmosphere without the beyond-table fallback)
 constexpr int kDispBit = 16;
 constexpr int kCurvBit = 32;
+// and the hits kernel that propagates all bunches, the one that decides, and
+// the one for large arrays
+constexpr int kDirectBit = 64;
+constexpr int kProbeBit = 128;
+constexpr int kLargeBit = 256;
 constexpr int kDispBlock = 128;
-inline int kernel_mode(int mode, const KParams &p) {
+inline int kernel_mode(int mode, const KParams &p, bool fp32) {
     int m = mode;
     if (p.trans && mode != MODE_YIELD) m |= kTransBit;
     if (p.fb_q > 0.0 && (mode == MODE_HITS || mode == MODE_TRACE)) m |= kFbBit;
     if (p.disp_k > 0) m |= kDispBit;
     if (p.earth_radius > 0.0) m |= kCurvBit;
+    else if (mode == MODE_HITS && fp32 && p.cull.words > kCullFewWords) m |= kLargeBit;
     return m;
 }
 // Zeros in the trace arrays, status -1.

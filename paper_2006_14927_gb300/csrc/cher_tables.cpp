@@ -573,7 +573,13 @@ cher_status build_grid(const cher_telescope *tel, int32_t n_tel, double theta_ma
 
 void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
     b.words = (n_tel + 31) / 32;
-    b.masks.assign(2 * size_t(kCullBins + 1) * b.words, 0u);
+    b.order.resize(n_tel);
+    for (int k = 0; k < n_tel; ++k) b.order[k] = k;
+    if (b.words > kCullFewWords)
+        std::stable_sort(b.order.begin(), b.order.end(),
+                         [&](int32_t p, int32_t q) { return tel[p].x < tel[q].x; });
+    const size_t nm = 2 * size_t(kCullBins + 1) * b.words;
+    b.masks.assign(nm + 2 * size_t(kCullBins + 1), 0u);
     for (int axis = 0; axis < 2; ++axis) {
         double lo = 1e300, hi = -1e300;
         for (int k = 0; k < n_tel; ++k) {
@@ -589,12 +595,16 @@ void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
         (axis ? b.y0 : b.x0) = -edge;
         (axis ? b.inv_by : b.inv_bx) = 0.5 * kCullBins / edge;
         uint32_t *m = b.masks.data() + axis * size_t(kCullBins + 1) * b.words;
+        uint32_t *count = b.masks.data() + nm + axis * size_t(kCullBins + 1);
         for (int k = 0; k < n_tel; ++k) {
-            const double at = ((axis ? tel[k].y : tel[k].x) - mid) / edge;      // in (-1, 1)
+            const cher_telescope &q = tel[b.order[k]];
+            const double at = ((axis ? q.y : q.x) - mid) / edge;      // in (-1, 1)
             const int bin = std::min(kCullBins - 1,
                                      static_cast<int>(0.5 * kCullBins * (at + 1.0)));
-            for (int e = bin + 1; e <= kCullBins; ++e)
+            for (int e = bin + 1; e <= kCullBins; ++e) {
                 m[size_t(e) * b.words + k / 32] |= 1u << (k % 32);
+                ++count[e];
+            }
         }
     }
 }
