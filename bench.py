@@ -100,15 +100,17 @@ FP64_FMA_PER_SM_CLK = 2         # GB300: 1/64 of the FP32 rate (ncu: 2 DFMA/cycl
 # share: the bound (without its tests of single telescopes); per drawn bunch:
 # the sub-step loop, Philox for one word (the last round's other half is not
 # needed) and the sector test.  The shares of drawn and propagated bunches were
-# counted on each workload.
+# counted with counters in a copy of the kernel at 2e6 steps of each workload
+# (FP32; FP64: the same to 2e-4); they hold for the kernel sources that hash to
+# what was counted, and without them the line has no fraction.
 OPS_PER_STEP_BOUND = 110
 OPS_PER_STEP_REACH = (OPS_PER_STEP_FP32["validity"] + OPS_PER_STEP_FP32["yield"] +
                       OPS_PER_STEP_FP32["philox_step_share"] + OPS_PER_STEP_BOUND)   # 179
 OPS_PER_DRAWN = 66
 BUNCH_SHARES = {                # drawn, propagated
-    "vertical_1tev": (0.4307, 0.02500),
-    "inclined_20tev": (0.6857, 0.02486),
-    "batched_256": (0.2129, 0.01424),
+    "vertical_1tev": (0.4307, 0.02500, "a1bb7d8fb58811a6"),
+    "inclined_20tev": (0.6860, 0.02489, "a1bb7d8fb58811a6"),
+    "batched_256": (0.2135, 0.01422, "a1bb7d8fb58811a6"),
 }
 
 # DRAM bytes (read + write) per step of one FP32 launch, from ncu captures
@@ -117,9 +119,9 @@ BUNCH_SHARES = {                # drawn, propagated
 # by its steps (the inputs, 64 B per step, dominate and scale with them).
 # Reported only while the kernel sources hash to what was profiled.
 TRAFFIC_PER_STEP = {
-    "vertical_1tev": (89.06, "fd01f26aca17b9e1"),      # 147.32 + 30.81 MB at 2e6 steps, 128 x 8
-    "inclined_20tev": (80.01, "fd01f26aca17b9e1"),     # 146.24 + 13.77 MB at 2e6 steps, 128 x 8
-    "batched_256": (80.87, "fd01f26aca17b9e1"),        # 144.29 + 17.45 MB at 2e6 steps, 128 x 8
+    "vertical_1tev": (89.04, "a1bb7d8fb58811a6"),      # 147.27 + 30.81 MB at 2e6 steps, 128 x 8
+    "inclined_20tev": (79.96, "a1bb7d8fb58811a6"),     # 146.15 + 13.76 MB at 2e6 steps, 128 x 8
+    "batched_256": (80.83, "a1bb7d8fb58811a6"),        # 144.37 + 17.28 MB at 2e6 steps, 128 x 8
 }
 KERNEL_SOURCES = ("cher_hits.cu", "cher_path.cuh", "cher_device.cuh", "cher_internal.h")
 
@@ -169,10 +171,16 @@ def fp64_roofline(bunches: float, steps: float, ms: float, sm_count: int, mhz: f
 def needed(rl: dict, wl: str, bunches: float, steps: float, ms: float):
     """The roofline of propagating every bunch (alu_roofline, fp64_roofline)
     with achieved and frac replaced by those of the operations the launch
-    needs; the former stay as all_bunches_*."""
+    needs (None where the shares were counted on other kernel sources); the
+    former stay as all_bunches_*."""
     if wl not in BUNCH_SHARES:
         return rl
-    drawn, prop = BUNCH_SHARES[wl]
+    drawn, prop, counted_on = BUNCH_SHARES[wl]
+    if _kernel_hash() != counted_on:
+        return {**rl, "achieved": None, "frac": None, "all_bunches_achieved": rl["achieved"],
+                "all_bunches_frac": rl["frac"],
+                "note": "the shares of drawn and propagated bunches were counted on other "
+                        "kernel sources"}
     if rl["bound"] == "alu":
         ops = OPS_PER_STEP_REACH * steps + (OPS_PER_DRAWN * drawn + OPS_PER_BUNCH * prop) * bunches
     else:

@@ -27,15 +27,19 @@
 // (yield, bound, telescopes) and in the drawn Philox words, not in the
 // propagation, and issue slots bound the FP32 kernel: on GB300, 2e6 steps,
 // 62-68 % of them used with 30 of 64 warps resident (64 registers; the rest is
-// waiting for the steps' and telescopes' loads), FP64 pipe 21-32 %, DRAM
+// waiting for the steps' and telescopes' loads), FP64 pipe 23-36 %, DRAM
 // 81-90 bytes a step (the step is 64, a crossing's record 40).  The FP64 kernel
 // is bound by its pipe (83 % busy: the yields' chains and the propagation).
 // Per launch, against the kernel that propagated every bunch:
-//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 283 us
-//   2e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1667 us
-//   3e6 steps, 60 deg, 100 spheres            FP32   685 -> 496 us
+//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 281 us
+//   2e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1722 us
+//   3e6 steps, 60 deg, 100 spheres            FP32   685 -> 490 us
 //   2e5 steps, vertical 100 GeV, 19 spheres   FP64  1477 -> 162 us
-//   3e5 steps with spectra                    FP32   234 -> 138 us
+//   3e5 steps with spectra                    FP32   234 -> 135 us
+// (1 - 2 % of that are the FP64 subtractions and the margin that keep the bound
+// right at any coordinates.)  Where rings pass many telescopes the bound costs
+// more than it saves, and launches over such arrays take the kernel that
+// propagates all bunches (k_probe, below).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -882,8 +886,9 @@ __device__ __forceinline__ void hits(const KParams &p) {
 }
 
 // One instantiation for every block size: 64 registers in FP32 (1024 threads
-// per SM), 128 in FP64.  With spectra (128-step blocks only) 72: seven CTAs per
-// SM without spills against eight with them, 144 -> 136 us at 3e5 steps.
+// per SM; none spilled but 4 bytes with the transmission draw or the fallback),
+// up to 148 in FP64.  With spectra (128-step blocks only) 72: seven CTAs per SM
+// with 24 - 36 bytes spilled against eight with more, 144 -> 136 us at 3e5 steps.
 template <class R, int MODE, bool TR, int FB, bool DS, int KIND>
 __global__ void __launch_bounds__(DS ? 128 : 512, std::is_same<R, float>::value ? (DS ? 7 : 2) : 1)
     k_hits(const __grid_constant__ KParams p) {

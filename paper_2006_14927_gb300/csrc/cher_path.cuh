@@ -1432,9 +1432,10 @@ __device__ __forceinline__ void flush_stat_signed(unsigned long long *stats, int
 // of the arrival line with the horizontal plane through the sphere centre.
 // All 32 lanes call it (hm = 0 on lanes without a crossing).  The photon
 // weight, record key, wavelength and arrival time at h_obs come from
-// weight_key(w, key, lambda, t), called on the hit path only.  The fallback
-// pass records through it; the fused kernel queues its crossings and
-// records them with flush_ring, the same steps one crossing per lane.
+// weight_key(w, key, lambda, t), called on the hit path only.  The hits kernels
+// of flat layers and the fallback pass record through it; the curved ones queue
+// their crossings and record them with flush_ring, the same steps one crossing
+// per lane.
 template <class R, class KW>
 __device__ __forceinline__ void record_hits(const KParams &p, const BunchOut<R> &o, unsigned hm,
                                             int s0, int gsel, KW weight_key, R np1o, int lane,
