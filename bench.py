@@ -108,9 +108,9 @@ OPS_PER_STEP_REACH = (OPS_PER_STEP_FP32["validity"] + OPS_PER_STEP_FP32["yield"]
                       OPS_PER_STEP_FP32["philox_step_share"] + OPS_PER_STEP_BOUND)   # 179
 OPS_PER_DRAWN = 66
 BUNCH_SHARES = {                # drawn, propagated
-    "vertical_1tev": (0.4307, 0.02500, "a1bb7d8fb58811a6"),
-    "inclined_20tev": (0.6860, 0.02489, "a1bb7d8fb58811a6"),
-    "batched_256": (0.2135, 0.01422, "a1bb7d8fb58811a6"),
+    "vertical_1tev": (0.4307, 0.02500, "19457bf171f9cbf8"),
+    "inclined_20tev": (0.6860, 0.02489, "19457bf171f9cbf8"),
+    "batched_256": (0.2135, 0.01422, "19457bf171f9cbf8"),
 }
 
 # DRAM bytes (read + write) per step of one FP32 launch, from ncu captures
@@ -119,9 +119,9 @@ BUNCH_SHARES = {                # drawn, propagated
 # by its steps (the inputs, 64 B per step, dominate and scale with them).
 # Reported only while the kernel sources hash to what was profiled.
 TRAFFIC_PER_STEP = {
-    "vertical_1tev": (89.04, "a1bb7d8fb58811a6"),      # 147.27 + 30.81 MB at 2e6 steps, 128 x 8
-    "inclined_20tev": (79.96, "a1bb7d8fb58811a6"),     # 146.15 + 13.76 MB at 2e6 steps, 128 x 8
-    "batched_256": (80.83, "a1bb7d8fb58811a6"),        # 144.37 + 17.28 MB at 2e6 steps, 128 x 8
+    "vertical_1tev": (89.20, "19457bf171f9cbf8"),      # 147.35 + 31.04 MB at 2e6 steps, 128 x 8
+    "inclined_20tev": (79.93, "19457bf171f9cbf8"),     # 146.14 + 13.71 MB at 2e6 steps, 128 x 8
+    "batched_256": (80.90, "19457bf171f9cbf8"),        # 144.36 + 17.45 MB at 2e6 steps, 128 x 8
 }
 KERNEL_SOURCES = ("cher_hits.cu", "cher_path.cuh", "cher_device.cuh", "cher_internal.h")
 

@@ -332,6 +332,8 @@ cher::KParams base_params(const cher_ctx *c, const cher_tracks *t, uint64_t seed
     p.cull.words = c->CB.words;
     p.cull.ox = c->CB.ox;
     p.cull.oy = c->CB.oy;
+    p.cull.oxf = static_cast<float>(c->CB.ox);
+    p.cull.oyf = static_cast<float>(c->CB.oy);
     p.cull.ex = static_cast<float>(c->CB.ex);
     p.cull.ey = static_cast<float>(c->CB.ey);
     // Rounding of coordinates, four of at most half an ulp each (2.4e-7 of

@@ -27,17 +27,16 @@
 // (yield, bound, telescopes) and in the drawn Philox words, not in the
 // propagation, and issue slots bound the FP32 kernel: on GB300, 2e6 steps,
 // 62-68 % of them used with 30 of 64 warps resident (64 registers; the rest is
-// waiting for the steps' and telescopes' loads), FP64 pipe 23-36 %, DRAM
+// waiting for the steps' and telescopes' loads), FP64 pipe 21-33 %, DRAM
 // 81-90 bytes a step (the step is 64, a crossing's record 40).  The FP64 kernel
 // is bound by its pipe (83 % busy: the yields' chains and the propagation).
 // Per launch, against the kernel that propagated every bunch:
-//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 281 us
-//   2e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1722 us
-//   3e6 steps, 60 deg, 100 spheres            FP32   685 -> 490 us
-//   2e5 steps, vertical 100 GeV, 19 spheres   FP64  1477 -> 162 us
-//   3e5 steps with spectra                    FP32   234 -> 135 us
-// (1 - 2 % of that are the FP64 subtractions and the margin that keep the bound
-// right at any coordinates.)  Where rings pass many telescopes the bound costs
+//   2e6 steps, vertical 1 TeV, 19 spheres     FP32   745 -> 279 us
+//   2e7 steps, 256 showers, 100 spheres       FP32  6870 -> 1704 us
+//   3e6 steps, 60 deg, 100 spheres            FP32   685 -> 488 us
+//   2e5 steps, vertical 100 GeV, 19 spheres   FP64  1477 -> 156 us
+//   3e5 steps with spectra                    FP32   234 -> 134 us
+// Where rings pass many telescopes the bound costs
 // more than it saves, and launches over such arrays take the kernel that
 // propagates all bunches (k_probe, below).
 #include <cuda_runtime.h>
@@ -123,15 +122,23 @@ struct Box {
     float sec_lo, sec_hi;         // bounds of 1 / cos(theta_o) over the step's bunches
 };
 
+// A step's coordinate from the middle of the array, which is a float: the FP32
+// path's ground points start from the rounded coordinate, so the difference is
+// formed from that (two FP64 subtractions a step cost 2 % of a launch).
+template <class R>
+__device__ __forceinline__ float from_middle(double x, double o, float of) {
+    if constexpr (std::is_same<R, float>::value) return __double2float_rn(x) - of;
+    else return __double2float_rn(x - o);
+}
+
 // Sets up a step's ring; REACH_ALL where the bound does not hold or a bunch
 // may be dropped on its way to the ground.  (Written without early returns:
 // the lanes of a group stay together.)
 template <int MODE, bool DS>
-__device__ __forceinline__ int ring_setup(const KParams &p, double x0d, double y0d, float dz0,
-                                          float L, float ux, float uy, float uz, float eta,
-                                          float sinc_lo, float sinc_hi, Ring &G, Near &N, Box &B) {
-    // from the middle of the array, and the rounding of coordinates
-    const float x0 = __double2float_rn(x0d - p.cull.ox), y0 = __double2float_rn(y0d - p.cull.oy);
+__device__ __forceinline__ int ring_setup(const KParams &p, float x0, float y0, float dz0, float L,
+                                          float ux, float uy, float uz, float eta, float sinc_lo,
+                                          float sinc_hi, Ring &G, Near &N, Box &B) {
+    // (x0, y0: from the middle of the array); the rounding of coordinates
     const float err = p.cull.err_m * (fmaxf(fabsf(x0), p.cull.ex) + fmaxf(fabsf(y0), p.cull.ey)) +
                       p.cull.err_0;
     const float su2 = ux * ux + uy * uy;
@@ -578,7 +585,8 @@ __device__ __forceinline__ void hits(const KParams &p) {
                     } else {
                         s_lo = s_hi = sqrtf(d2f_rn(y.s2));
                     }
-                    kind = ring_setup<MODE, DS>(p, __ldg(p.x0 + i), __ldg(p.y0 + i),
+                    kind = ring_setup<MODE, DS>(p, from_middle<R>(__ldg(p.x0 + i), p.cull.ox, p.cull.oxf),
+                                                from_middle<R>(__ldg(p.y0 + i), p.cull.oy, p.cull.oyf),
                                                 __double2float_rn(z0) - p.f.h_obs,
                                                 __double2float_rn(len), ux, uy, uzf,
                                                 eta, s_lo, s_hi,
@@ -943,7 +951,9 @@ __global__ void __launch_bounds__(256) k_probe(const __grid_constant__ KParams p
         Ring G;
         Near N;
         Box B;
-        int kind = ring_setup<MODE_HITS, DS>(p, x0, y0, __double2float_rn(z0) - p.f.h_obs,
+        int kind = ring_setup<MODE_HITS, DS>(p, from_middle<float>(x0, p.cull.ox, p.cull.oxf),
+                                             from_middle<float>(y0, p.cull.oy, p.cull.oyf),
+                                             __double2float_rn(z0) - p.f.h_obs,
                                              __double2float_rn(len), ux, uy, uz, y.eta, s_lo, s_hi,
                                              G, N, B);
         int tests = 0, near = 0, w0 = 0, w1 = p.cull.words;

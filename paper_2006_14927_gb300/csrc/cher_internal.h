@@ -65,9 +65,9 @@ cher_status build_grid(const cher_telescope *tel, int32_t n_tel, double theta_ma
                        HostGrid &g);
 // Prefix masks of the telescopes' centres over kCullBins bins per axis
 // (KParams::cull), and the largest slopes of ax over the table's cells.
-// Coordinates are taken from the middle (ox, oy) of the centres' box, whose
-// half sizes are ex, ey: single precision resolves the array wherever the
-// caller's coordinates have their origin.
+// Coordinates are taken from the middle (ox, oy, each a float) of the centres'
+// box, whose half sizes are ex, ey: single precision resolves the array wherever
+// the caller's coordinates have their origin.
 struct HostBins {
     int32_t words = 0;
     double ox = 0, oy = 0, ex = 0, ey = 0;
@@ -147,6 +147,7 @@ struct KParams {
     struct Cull {
         const float2 *tab32;
         double ox, oy;
+        float oxf, oyf;                   // (the same)
         float ex, ey, err_m, err_0;
         float ax_sq, ax_sh;
         int words;

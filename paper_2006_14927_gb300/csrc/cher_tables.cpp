@@ -587,7 +587,8 @@ void build_center_bins(const cher_telescope *tel, int32_t n_tel, HostBins &b) {
             lo = std::min(lo, v);
             hi = std::max(hi, v);
         }
-        const double mid = 0.5 * lo + 0.5 * hi, half = 0.5 * hi - 0.5 * lo;
+        const double mid = static_cast<float>(std::clamp(0.5 * lo + 0.5 * hi, -3e38, 3e38));
+        const double half = std::max(mid - lo, hi - mid);
         (axis ? b.oy : b.ox) = mid;
         (axis ? b.ey : b.ex) = half;
         // room on both sides for single-precision bin indices
