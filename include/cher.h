@@ -204,7 +204,8 @@ typedef struct cher_output {
 
 /* The whole hot path (a1-a5) for n steps in one launch: a persistent kernel
  * whose warps (in a curved atmosphere, CTAs) pull groups of steps from an
- * atomic queue in the context's scratch word.  Asynchronous on `stream`; the return value
+ * atomic queue in the context's scratch word (over crowded arrays a short
+ * kernel first chooses between two of them, and the other ends at once).  Asynchronous on `stream`; the return value
  * reports argument checks and the launch only.  Errors: CHER_EINVAL,
  * CHER_ESTATE, CHER_ERANGE (n > 2^40), CHER_ECUDA. */
 cher_status cher_generate_propagate(cher_ctx *ctx, const cher_tracks *tracks,
